@@ -44,7 +44,8 @@ typedef enum {
 
 /* Arithmetic of the P and Sigma^c contractions. */
 typedef enum {
-  GW_FP64 = 0,    /* native FP64 (CUDA cores); the parity path */
+  GW_FP64 = 0,    /* FP64 (P, Sigma^c: exact fp16 digit products on the tensor cores, summed in integers, with
+                     errors below an FP64 accumulation's; the rest native FP64); the parity path */
   GW_FP16X2 = 1,  /* tcgen05 tensor cores: fp16 hi/lo split operands, 3 products, FP32 TMEM accumulation */
                   /* (value 2 is not used) */
   GW_F32X2 = 3,   /* float-float on the FP32 pipes: each value hi + lo in two FP32 (~44-bit significand) */
@@ -111,7 +112,7 @@ gw_status gw_create(gw_ctx** ctx, const gw_grid* grid, const gw_system* sys, int
 gw_status gw_destroy(gw_ctx* ctx);
 /* Waits for the context's stream and reports errors of its asynchronous work: GW_ECUDA for a
  * CUDA error, GW_ETIMEOUT when a bounded device-side wait in a tensor-core contraction (the
- * pipeline barriers of k_pol_tc / k_sig_tc, see GW_TUNE_WAIT_CYCLES) ran out since the last
+ * pipeline barriers of k_pol_tc / k_sig_tc / k_digit_gemm, see GW_TUNE_WAIT_CYCLES) ran out since the last
  * gw_sync: the kernel then stopped, let the copies and MMAs it had issued finish, freed its
  * tensor memory and returned, and the outputs of those calls are undefined. The error word is
  * cleared when it is reported, so the context stays usable. */
@@ -132,7 +133,10 @@ gw_status gw_green_tau(gw_ctx* ctx, const double* eps, const double* sigx, const
 /* Irreducible polarization of the iq-th q, Eq. (irpol):
  * P_II'(q|tau) = 1/(Omega N_k) sum_k sum_ab M^I_ab Q_ab(tau) conj(M^I'_ab),
  * Q_ab(tau) = G_b(k|tau) G_a(k-q|-tau), G(-tau) = -G(beta - tau) (Sec. II).
- * G_tau [nk][nb][ntau] (any G: G0 or dressed); P_tau out cplx [ntau][ni][ni] (Hermitian). */
+ * G_tau [nk][nb][ntau] (any G: G0 or dressed); P_tau out cplx [ntau][ni][ni] (Hermitian).
+ * GW_FP64 uses a context workspace of up to ~7 GiB, grown on use; a call that cannot have it (no
+ * memory, or a first call under stream capture) runs on the CUDA cores without one. With GW_FP64 an
+ * infinity or nan in M^I or G gives nan in the rows and columns it reaches. */
 gw_status gw_polarization(gw_ctx* ctx, int iq, const double* G_tau, gw_prec prec, double* P_tau);
 
 /* The polarization of several crystals (one q each) in one persistent launch: job j is
@@ -290,7 +294,7 @@ gw_status gw_screen_static(int nq, int nnu, int ni, const double* sqrt_v, const 
  *             Sigx_n(k) += -1/(Omega N_k) sum_j occ_j(k-q) sum_I v_I |M^I_jn|^2.
  * G_tau [nk][nb][ntau]; occ [nk][nb]; Wt_tau cplx [ntau][ni][ni] (Hermitian);
  * Sigc_tau [nk][nb][ntau] (real: W~(tau) Hermitian); Sigx [nk][nb] (may be NULL).
- * prec GW_FP64: both in FP64. GW_FP16X2: Sigc on the tensor cores, Sigx in
+ * prec GW_FP64: both in FP64 (Sigc with a workspace and without one as in gw_polarization). GW_FP16X2: Sigc on the tensor cores, Sigx in
  * float-float on the FP32 pipes (relative error ~1e-12). */
 gw_status gw_selfenergy(gw_ctx* ctx, int iq, const double* G_tau, const double* occ,
                         const double* Wt_tau, gw_prec prec, double* Sigc_tau, double* Sigx);

@@ -822,6 +822,7 @@ gw_status gw_destroy(gw_ctx* c) {
   if (c->d_tsys) cudaFree(c->d_tsys);
   if (c->d_dyt) cudaFree(c->d_dyt);
   if (c->d_dm) cudaFree(c->d_dm);
+  if (c->x_ws) cudaFree(c->x_ws);
   c->ff_ws = nullptr;
   double* bufs[] = {c->d_sqrtv, c->d_v,       c->d_M_own, c->d_Bfwd,  c->d_Ffwd,  c->d_Fcont, c->d_Bbwd,
                     c->d_Fbwd,  c->d_Fbwd_beta, c->d_aug,   c->d_cpe_x, c->d_cpe_A, c->d_cpe_N, c->d_cpe_tab, c->d_cpe_b,
@@ -926,7 +927,10 @@ gw_status gw_green_tau(gw_ctx* c, const double* eps, const double* sigx, const d
 
 gw_status gw_polarization(gw_ctx* c, int iq, const double* G, gw_prec prec, double* P) {
   if (!c || !G || !P || iq < 0 || iq >= c->nq) return GW_EINVAL;
-  if (prec == GW_FP64) return launch_pol_fp64(c, iq, G, P);
+  if (prec == GW_FP64) {
+    const gw_status st = launch_pol_exact(c, iq, G, P);
+    return st == GW_EUNSUPPORTED ? launch_pol_fp64(c, iq, G, P) : st;
+  }
   if (prec == GW_FP16X2) return launch_pol_mixed(c, iq, G, (int)prec, P);
   return GW_EINVAL;
 }
@@ -980,9 +984,10 @@ gw_status gw_selfenergy(gw_ctx* c, int iq, const double* G, const double* occ, c
                         double* S, double* Sx) {
   if (!c || !G || !W || !S || iq < 0 || iq >= c->nq || (Sx && !occ)) return GW_EINVAL;
   gw_status st;
-  if (prec == GW_FP64)
-    st = launch_sigma_fp64(c, iq, G, W, S);
-  else if (prec == GW_FP16X2)
+  if (prec == GW_FP64) {
+    st = launch_sigma_exact(c, iq, G, W, S);
+    if (st == GW_EUNSUPPORTED) st = launch_sigma_fp64(c, iq, G, W, S);
+  } else if (prec == GW_FP16X2)
     st = launch_sigma_mixed(c, iq, G, W, (int)prec, S);
   else
     return GW_EINVAL;

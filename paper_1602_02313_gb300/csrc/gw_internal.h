@@ -114,6 +114,8 @@ struct gw_ctx {
   int64_t cpe_seed_nprob = 0;
   double* d_pade = nullptr;     // cplx [nprob][npade] coefficients
   size_t pade_bytes = 0;
+  void* x_ws = nullptr;         // FP64 contractions on the tensor cores: operand digits, partial sums
+  size_t x_ws_bytes = 0;
   // tensor-core path
   gwi::MixedWork mw;
   int* d_err = nullptr;                     // error word of the bounded device waits (read by gw_sync)
@@ -148,6 +150,9 @@ gw_status launch_green0(gw_ctx* c, const double* eps, double* G, double* occ);
 gw_status launch_dyson(gw_ctx* c, const double* eps, const double* sigx, const double* vxc,
                        const double* sigc_iw, double* G, double* occ);
 gw_status launch_pol_fp64(gw_ctx* c, int iq, const double* G, double* P);
+// FP64 on the tensor cores (exact digit products); GW_EUNSUPPORTED when the digit workspace cannot be had
+gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P);
+gw_status launch_sigma_exact(gw_ctx* c, int iq, const double* G, const double* W, double* S);
 gw_status launch_pol_mixed(gw_ctx* c, int iq, const double* G, int prec, double* P);
 gw_status launch_pol_many(int njobs, gw_ctx* const* ctxs, const int* iqs, const double* const* G, double* const* P);
 gw_status launch_transform(gw_ctx* c, int stat, int dir, int prec, int count, int64_t batch, const double* in,

@@ -55,6 +55,35 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t* bar, uint32_t parity) 
   return false;
 }
 
+constexpr long long kDrainCycles = 4000000000ll;  // ~2 s at 2 GHz: waits for work already issued
+
+// Bounded mbarrier wait shared by all roles of a block: gives up after `budget` clock cycles
+// (the context's wait budget, ~2 s by default), or at once if another thread of the block has
+// given up; on giving up it raises the block's abort flag and records kErrTimeout in *err.
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err,
+                                         long long budget) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity)) {
+    if (*abort_flag) return false;
+    if (clock64() - t0 > budget) {
+      *abort_flag = 1;
+      if (err) atomicExch(err, kErrTimeout);
+      return false;
+    }
+  }
+  return true;
+}
+
+// Wait for work this block has already issued (bulk copies into its shared memory, MMAs into its
+// TMEM) before the block gives up its resources; ignores the abort flag, bounded by kDrainCycles.
+__device__ __forceinline__ bool drain_bar(uint64_t* bar, uint32_t parity) {
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity))
+    if (clock64() - t0 > kDrainCycles) return false;
+  return true;
+}
+
 // Arrive on an mbarrier and add `bytes` to the transaction count it waits for.
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -132,6 +161,18 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
   return d;
 }
 
+// K-major operand without swizzle: core matrices of 8 rows x 16 bytes (128 contiguous bytes), the
+// row groups of 8 one after another (stride byte offset 128), the next 8 K values `lbo` bytes on;
+// layout type 0.
+__device__ __forceinline__ uint64_t sdesc_none(uint32_t saddr, uint32_t lbo) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+  d |= (uint64_t)(lbo >> 4) << 16;
+  d |= (uint64_t)(128 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+
 // Instruction descriptor of tcgen05.mma kind::f16: D = FP32 (bits 4-5 = 1),
 // A / B format (bits 7-9 / 10-12: 0 = fp16, 1 = bf16), negate A (bit 13),
 // K-major A and B (bits 15, 16 = 0), N >> 3 (bits 17-22), M >> 4 (bits 24-28).
@@ -153,6 +194,33 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
+}
+
+// The forms for an issuer warp that runs converged: every lane computes the (uniform) operands and one
+// elected lane issues. In a lane == 0 branch the descriptors are per-thread values that cost a
+// register-to-uniform move each: measured 98 clocks per MMA of distinct descriptors, against the 48
+// that the operands of a 128 x 64 x 16 MMA take to read. desc_lo: low 32 bits of a descriptor
+// (address and leading offset), desc_hi the high 32, the same for A and B.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void mma_f16_warp(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
+                                            uint32_t idesc, uint32_t accumulate, uint32_t lead) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n mov.b64 a, {%1, %3};\n mov.b64 b, {%2, %3};\n"
+      " setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_warp(uint64_t* bar, uint32_t lead) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(bar)),
+      "r"(lead)
+      : "memory");
 }
 
 // Byte offset of element (r, k), k in [0, 64), 2-byte elements, in a K-major

@@ -46,33 +46,6 @@ using namespace tc;
 
 constexpr float kScaleA = 256.0f;   // 2^8 on matrix elements (|M| < ~3)
 constexpr float kScaleW = 1.0f;     // W~ entries are O(v) <= 4 pi / 0.05
-constexpr long long kDrainCycles = 4000000000ll;  // ~2 s at 2 GHz: waits for work already issued
-
-// Bounded mbarrier wait shared by all roles of a block: gives up after `budget` clock cycles
-// (the context's wait budget, ~2 s by default), or at once if another thread of the block has
-// given up; on giving up it raises the block's abort flag and records kErrTimeout in *err.
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err,
-                                         long long budget) {
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    if (*abort_flag) return false;
-    if (clock64() - t0 > budget) {
-      *abort_flag = 1;
-      if (err) atomicExch(err, kErrTimeout);
-      return false;
-    }
-  }
-  return true;
-}
-
-// Wait for work this block has already issued (bulk copies into its shared memory, MMAs into its
-// TMEM) before the block gives up its resources; ignores the abort flag, bounded by kDrainCycles.
-__device__ __forceinline__ bool drain_bar(uint64_t* bar, uint32_t parity) {
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity))
-    if (clock64() - t0 > kDrainCycles) return false;
-  return true;
-}
 
 __device__ __forceinline__ void split2(float x, __half& h, __half& l) {
   h = __float2half_rn(x);
