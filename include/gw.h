@@ -156,7 +156,8 @@ gw_status gw_polarization_many(int njobs, gw_ctx* const* ctxs, const int* iqs, c
 /* Imaginary time <-> Matsubara transforms (Eq. trans and its bosonic / inverse
  * counterparts), fixed matrices (built in extended precision, stored FP64) applied as
  * batched matvecs. prec: GW_FP64 (native FP64), or GW_F32X2 for the two bosonic
- * directions (float-float arithmetic, relative error ~1e-13; the mixed chain's choice);
+ * directions (exact digit products on the tensor cores, relative error ~1e-13 where the map cancels;
+ * the mixed chain's choice; native FP64 when its digit workspace, up to ~120 MB, cannot be had);
  * anything else returns GW_EUNSUPPORTED.
  *  BOSE  TAU_TO_IW : in cplx [ntau][batch]        -> out cplx [nnu][batch]
  *  BOSE  IW_TO_TAU : in cplx [nnu][m][m] of a Hermitian-matrix function (batch = m)
@@ -171,8 +172,7 @@ gw_status gw_tau_to_freq(gw_ctx* ctx, gw_stat stat, gw_dir dir, int64_t batch, c
  * one after another (in [count][...in of one transform], out [count][...out of one]); the
  * bosonic directions run them in one grid (q points of a block of the chain), the fermionic
  * ones as one batch of count * batch rows. Results are those of count separate calls.
- * 1 <= count <= 65535, else GW_EINVAL. Float-float inputs are converted through a context
- * workspace in chunks of at most 2 GiB. */
+ * 1 <= count <= 65535, else GW_EINVAL. */
 gw_status gw_tau_to_freq_many(gw_ctx* ctx, gw_stat stat, gw_dir dir, int count, int64_t batch, const double* in,
                               gw_prec prec, double* out);
 

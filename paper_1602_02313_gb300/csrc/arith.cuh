@@ -1,4 +1,4 @@
-// Complex arithmetic policies shared by the FP64-bound kernels (screening, transforms).
+// Complex arithmetic policies of the FP64-bound kernels (screening; Fp64 also the transforms).
 //  * Fp64 : double2 values, FP64 fused multiply-adds.
 //  * F32  : float2 values, FP32 fused multiply-adds (rounding error ~6e-8 per operation; for
 //           the dielectric inverse of the mixed chain, whose input P already carries the
@@ -8,9 +8,8 @@
 //           it joins the accumulator through an error-free two-sum (Knuth), the errors
 //           collect in the accumulator's low word. All of it runs on the FP32 pipes, which
 //           on GB300 issue about 64 times more operations per clock than the FP64 ones.
-// Both expose: S (stored value), Acc (accumulator), from/to double, zero, azero, is_zero,
-// mac (acc += l u, complex), rmac (real parts: acc.re += a x, acc.im += a y for real a),
-// val (accumulator -> value), sub (b - acc), inv (complex reciprocal).
+// All expose: S (stored value), Acc (accumulator), from/to double, zero, azero, is_zero,
+// mac (acc += l u, complex), val (accumulator -> value), sub (b - acc), inv (complex reciprocal).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -40,14 +39,12 @@ struct Fp64 {
   __device__ static S val(Acc a) { return a; }
   __device__ static S sub(S b, Acc a) { return make_double2(b.x - a.x, b.y - a.y); }  // b - a
   __device__ static S inv(S v) { return cinv_d(v); }
-  using R = double;  // stored real coefficient
-  __device__ static R rfrom(double x) { return x; }
   __device__ static S add(S a, S b) { return make_double2(a.x + b.x, a.y + b.y); }
   __device__ static S dif(S a, S b) { return make_double2(a.x - b.x, a.y - b.y); }
   __device__ static S half(S a) { return make_double2(0.5 * a.x, 0.5 * a.y); }
   __device__ static S mul_mi(S a) { return make_double2(a.y, -a.x); }  // -i a
   // acc.re += A g.re + B g.im, acc.im += A h.re + B h.im
-  __device__ static void rmac2(Acc& acc, R A, R B, S g, S h) {
+  __device__ static void rmac2(Acc& acc, double A, double B, S g, S h) {
     acc.x = fma(A, g.x, fma(B, g.y, acc.x));
     acc.y = fma(A, h.x, fma(B, h.y, acc.y));
   }
@@ -138,42 +135,6 @@ struct Ff32 {
     const double2 d = to(v);
     const double2 r = cinv_d(d);
     return from(r.x, r.y);
-  }
-  struct __align__(8) R {
-    float h, l;
-  };
-  __device__ static R rfrom(double x) {
-    R r;
-    cvt::d2ff(x, r.h, r.l);
-    return r;
-  }
-  __device__ __forceinline__ static void ffadd(float ah, float al, float bh, float bl, float& h, float& l) {
-    const float s = ah + bh;
-    const float v = s - ah;
-    const float err = (ah - (s - v)) + (bh - v);
-    h = s;
-    l = err + (al + bl);
-    renorm(h, l);
-  }
-  __device__ static S add(S a, S b) {
-    S r;
-    ffadd(a.rh, a.rl, b.rh, b.rl, r.rh, r.rl);
-    ffadd(a.ih, a.il, b.ih, b.il, r.ih, r.il);
-    return r;
-  }
-  __device__ static S dif(S a, S b) {
-    S r;
-    ffadd(a.rh, a.rl, -b.rh, -b.rl, r.rh, r.rl);
-    ffadd(a.ih, a.il, -b.ih, -b.il, r.ih, r.il);
-    return r;
-  }
-  __device__ static S half(S a) { return {0.5f * a.rh, 0.5f * a.rl, 0.5f * a.ih, 0.5f * a.il}; }
-  __device__ static S mul_mi(S a) { return {a.ih, a.il, -a.rh, -a.rl}; }
-  __device__ static void rmac2(Acc& acc, R A, R B, S g, S h) {
-    ffmac(acc.rh, acc.rl, A.h, A.l, g.rh, g.rl);
-    ffmac(acc.rh, acc.rl, B.h, B.l, g.ih, g.il);
-    ffmac(acc.ih, acc.il, A.h, A.l, h.rh, h.rl);
-    ffmac(acc.ih, acc.il, B.h, B.l, h.ih, h.il);
   }
 };
 

@@ -1,25 +1,4 @@
-// FP64 contractions on the tensor cores by error-free splitting (Ozaki, Ogita, Oishi, Rump,
-// Numer. Algorithms 59, 95 (2012); on fp16 tensor cores: Mukunoki, Ozaki, Ogita, Imamura, ISC 2020).
-//
-// GB300's FP64 pipes run at ~1 TFLOP/s, its fp16 tensor cores at ~1900. Every operand row is scaled
-// by a power of two to |x| < 1 and written as a 56-bit fixed-point number of seven balanced 8-bit
-// digits, x = 2^e sum_i d_i 2^(-7 - 8 i), |d_i| <= 128, each digit an exact fp16 value. A product of
-// two rows is then sum_s 2^(-14 - 8 s) L_s with L_s = sum_k sum_(i + j = s) a_i b_j, an integer. The
-// levels s = 0 .. 6 (28 digit products) are formed on the tensor cores, one FP32 accumulator in
-// tensor memory per level, over blocks of 192 k: |L_s| <= (s + 1) 192 2^14 < 2^24 for s <= 4, so the
-// FP32 sums are exact there (at s = 5, 6 an extreme coherent row could round, by 2^-54 of the sum of
-// |a b|). The blocks' levels are added up in 64-bit integers and become one double per element at
-// the end. What is lost is the rounding of each operand to 2^-56 of its row's largest value and the
-// levels above 6: smaller than the rounding errors an FP64 accumulation of the same sum makes (the
-// measured errors against 64-bit sums are below the CUDA-core kernels' over all tested sizes).
-// Rows that hold an infinity or a nan give nan.
-//
-// Tile 128 x 64: the seven levels of 64 columns take 448 of the 512 TMEM columns. A 128 x 64 x 16 MMA
-// takes 48 clocks (its operands' 6 KB at 128 bytes per clock of shared memory; 32 of arithmetic), so
-// the bound is 28 x 48 clocks per chunk of 16 k and SM. Measured, Nk 27, Nb 32, NI 128, 32 tau: 0.72 ms
-// per 16 tau, 67 clocks per MMA with the levels' readout, which overlaps the next block's MMAs level
-// by level; P of one q 84.5 -> 2.2 ms, Sigma^c of one q at Nk 8, Nb 32, NI 128, 32 tau 33.3 -> 0.80 ms.
-// It is the faster form at every size measured, down to Nk 2, Nb 4, NI 32, 16 tau (70 -> 62 us).
+// FP64 contractions of the GW cycle as exact digit products on the tensor cores (digit_gemm.cuh).
 //
 // polarization, Eq. (irpol): E = Re P + Im P = X Y^T (the real cover of the Hermitian P used by the
 //   mixed path), rows of X = (tau, I): [w (re + im) | w (im - re)], rows of Y = I: [re | im]. One
@@ -27,385 +6,106 @@
 // self-energy, Eq. (sigc): d_p(tau) = 2 sum_J (re_p Y1 + im_p Y2)[p][J], [Y1 | Y2] = A B^T with
 //   A = [re | im] of the pair rows p and B built from the upper triangle of the Hermitian part of
 //   W~(tau); the dot with M runs in the epilogue in FP64.
-#include <cuda_fp16.h>
-#include <cuda_runtime.h>
-
+// Measured: P of one q at Nk 27, Nb 32, NI 128, 32 tau 84.5 -> 2.2 ms, Sigma^c of one q at Nk 8, Nb 32,
+// NI 128, 32 tau 33.3 -> 0.80 ms against the CUDA-core kernels; faster at every size measured, down to
+// Nk 2, Nb 4, NI 32, 16 tau (70 -> 62 us).
 #include <algorithm>
 
-#include "gw_internal.h"
-#include "tc_common.cuh"
+#include "digit_gemm.cuh"
 
 namespace gwi {
 
 namespace {
 
-using namespace tc;
-
-constexpr int XS_N = 7;                       // digits per operand
-constexpr int XK = 16;                        // K values per chunk: one MMA step
-constexpr int X_BLK = 12;                     // chunks per accumulation block (192 k)
-constexpr int XN = 64;                        // output columns per tile: 7 levels x 64 = 448 TMEM columns
-constexpr int XA_SL = 128 * 32, XB_SL = XN * 32;  // bytes of one digit of an operand chunk
-constexpr int XA_BYTES = XS_N * XA_SL, XB_BYTES = XS_N * XB_SL;
-constexpr int XST_BYTES = XA_BYTES + XB_BYTES;    // 42 KB per stage
-constexpr int X_ST = 5;                       // stages: a chunk's copy has four chunks' MMAs to land in
-constexpr int X_EPI = 16;                     // epilogue warps: 4 per TMEM lane quadrant, 16 columns each
-constexpr int X_THREADS = (X_EPI + 2) * 32;
-constexpr int kBadExp = 1 << 20;              // row exponent of a row that is not finite
-
-// ------------------------------------------------------------------ fixed point and digits
-// |x| in units of 2^e, as a float that is not smaller (x finite, |x| < 2^(e + 126)); 0 for x = 0.
-__device__ __forceinline__ float norm_up(double x, int e) {
-  const uint32_t hi = (uint32_t)(__double_as_longlong(x) >> 32) & 0x7FFFFFFFu;
-  if ((hi | (uint32_t)__double_as_longlong(x)) == 0) return 0.f;
-  const int ef = (int)(hi >> 20);
-  if (ef == 0) return __uint_as_float(1u << 23);
-  const int k = ef - 1023 - e;
-  if (k < -125) return __uint_as_float(1u << 23);
-  return __uint_as_float((((uint32_t)(k + 127) << 23) | ((hi & 0xFFFFFu) << 3)) + 8u);
-}
-// smallest e with |x| < 2^e for every x whose |high word| is at most h
-__device__ __forceinline__ int exp_of(uint32_t h) { return h >= 0x7FF00000u ? kBadExp : (int)(h >> 20) - 1022; }
-
-// rint(x 2^(55 - e)), |x| < 2^e: a 56-bit integer (0 for a row that is not finite)
-__device__ __forceinline__ long long to_fix(double x, int e) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const int ef = (int)(b >> 52) & 2047;
-  const uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (ef ? 1ull << 52 : 0ull);
-  const int sh = (ef ? ef : 1) - 1020 - e;
-  uint64_t t;
-  if (sh >= 0)
-    t = sh < 3 ? m << sh : 0;
-  else
-    t = sh > -55 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0;
-  return (long long)b < 0 ? -(long long)t : (long long)t;
-}
-
-// sign, exponent field and left-justified 64-bit mantissa (0 for zero) of a double
-struct Fl64 {
-  uint64_t m;
-  int e;  // |x| = m 2^(e - 1086)
-};
-__device__ __forceinline__ Fl64 fl64(double x) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const int ef = (int)(b >> 52) & 2047;
-  Fl64 r;
-  r.m = ((b & 0xFFFFFFFFFFFFFull) | (ef ? 1ull << 52 : 0ull)) << 11;
-  r.e = ef ? ef : 1;
-  return r;
-}
-// rint(|x| |w| 2^(55 - e)), |x w| < 2^e (0 where the shift leaves the word: a row that is not finite)
-__device__ __forceinline__ uint64_t mul_fix(const Fl64& x, const Fl64& w, int e) {
-  const uint64_t h = __umul64hi(x.m, w.m);  // |x w| = h 2^(xe + we - 2108)
-  const int sr = 2053 - x.e - w.e + e;
-  return sr >= 1 && sr < 64 ? (h >> sr) + ((h >> (sr - 1)) & 1) : 0;
-}
-
-// the digits of 8 values as 16 bytes of fp16 per slice: the six lower digits are the bytes of the
-// biased integer minus 128 (0x6400 | byte is the half 1024 + byte)
-__device__ __forceinline__ void digits8(const long long (&t)[8], uint4 (&out)[XS_N]) {
-  uint32_t w[XS_N][4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint64_t u0 = (uint64_t)(t[2 * q] + 0x0000808080808080ll), u1 = (uint64_t)(t[2 * q + 1] + 0x0000808080808080ll);
-    const uint32_t l0 = (uint32_t)u0, l1 = (uint32_t)u1, h0 = (uint32_t)(u0 >> 32), h1 = (uint32_t)(u1 >> 32);
-    const __half2 bias = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));  // 1152
-    auto put = [&](int s, uint32_t r) {
-      const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&r), bias);
-      w[s][q] = *reinterpret_cast<const uint32_t*>(&d);
-    };
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      put(6 - j, (__byte_perm(l0, l1, j | ((4 + j) << 8)) & 0x00FF00FFu) | 0x64006400u);
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-      put(2 - j, (__byte_perm(h0, h1, j | ((4 + j) << 8)) & 0x00FF00FFu) | 0x64006400u);
-    const uint32_t t0 = (uint32_t)(((int)h0 >> 16) + 128), t1 = (uint32_t)(((int)h1 >> 16) + 128);
-    put(0, (t0 | (t1 << 16)) + 0x64006400u);
-  }
-#pragma unroll
-  for (int s = 0; s < XS_N; ++s) out[s] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-}
-
-// 8 consecutive K values (k8 = 0, 1 of the chunk) of one row of an operand chunk [digit][k8][rows][16 B]
-template <int ROWS>
-__device__ __forceinline__ void put8(unsigned char* chunk, int row, int k8, const long long (&t)[8]) {
-  uint4 d[XS_N];
-  digits8(t, d);
-  unsigned char* o = chunk + (k8 * ROWS + row) * 16;
-#pragma unroll
-  for (int s = 0; s < XS_N; ++s) *reinterpret_cast<uint4*>(o + s * ROWS * 32) = d[s];
-}
-
-__device__ __forceinline__ uint32_t abs_hi(double x) {
-  return (uint32_t)(__double_as_longlong(x) >> 32) & 0x7FFFFFFFu;
-}
-__device__ __forceinline__ uint32_t warp_max(uint32_t v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
-// y 2^e rounded to nearest even, on the integer pipes (a conversion from 64-bit integers and a
-// product would take two slots of the FP64 pipe, which two such slots per element already fill);
-// nan when a row of the element is not finite
-__device__ __forceinline__ double fix_to_double(long long y, int e) {
-  if (e > kBadExp / 2) return __longlong_as_double(0x7FF8000000000000ll);
-  if (y == 0) return 0.0;
-  const uint64_t a = y < 0 ? 0ull - (uint64_t)y : (uint64_t)y;
-  const int lz = __clzll((long long)a), ex = 1023 + 63 - lz + e;
-  if (ex < 1 || ex > 2045) return scalbn((double)y, e);
-  const uint64_t m = a << lz, r = m >> 11, rest = m & 2047;
-  const uint64_t up = rest > 1024 || (rest == 1024 && (r & 1)) ? 1 : 0;
-  const uint64_t b = ((uint64_t)(ex - 1) << 52) + r + up;  // r carries the implicit bit
-  return __longlong_as_double((long long)(b | ((uint64_t)y & 0x8000000000000000ull)));
-}
-
-// ------------------------------------------------------------------ the digit GEMM
-struct XSmem {
-  uint64_t full[X_ST], empty[X_ST], done, lvl[XS_N], fin, never;
-  uint32_t tslot;
-  int abort_flag, no_dealloc;
-  double red[3][128];
-};
-
-// Store mode: unit = (K split, M tile, N tile), C[split][row][n] = sum over the split's chunks.
-// Dot mode: unit = (M tile, tau), all N tiles jt (32 columns J of Y1 beside the same J of Y2) over
-// the K chunks I <= J, dotted with M: D[row][tau].
-struct XJob {
-  const unsigned char* A;  // [M tile][chunk][digit][k8][128 x 16 B]
-  const unsigned char* B;  // [tau][N tile][chunk][digit][k8][64 x 16 B]
-  const int *ea, *eb;      // row exponents: A [rows], B [tau][ncols] ([tau][J] in dot mode)
-  int mt, nt, chunks, nsplit, rows, ncols;
-  double* C;
-  const double2* M;        // dot mode: M[k][J][p] of the job's first row
-  int np, ni, ntau, tau0, ntau_all, tgrp;
-  int sh;                  // bits of the 96-bit sums dropped at the end: K 2^14 2^48 < 2^(62 + sh)
-  double* D;
-};
-
-template <bool DOT>
-struct XUnit {
-  int m, b, s, n0, n1;
-  __device__ XUnit(const XJob& J, int u) {
-    if (DOT) {  // tau in groups of tgrp, inside a group the M tiles, inside those the group's tau
-      const int per = J.mt * J.tgrp, g = u / per, r = u % per;
-      const int gt = min(J.tgrp, J.ntau - g * J.tgrp);
-      m = r / gt;
-      b = g * J.tgrp + r % gt;
-      s = 0;
-      n0 = 0;
-      n1 = J.nt;
-    } else {
-      n0 = u % J.nt;
-      n1 = n0 + 1;
-      m = (u / J.nt) % J.mt;
-      s = u / (J.nt * J.mt);
-      b = 0;
-    }
-  }
-  __device__ void range(const XJob& J, int n, int& c0, int& c1) const {
-    if (DOT) {
-      c0 = 0;
-      c1 = 4 * (n + 1);
-    } else {
+// ------------------------------------------------------------------ what the GEMM does with its tiles
+// Polarization: unit = (K split, M tile, N tile), C[split][row][n] = sum over the split's chunks.
+struct OpStore {
+  struct Job {
+    const unsigned char *A, *B;  // [M tile][chunk], [N tile][chunk]
+    const int *ea, *eb;          // row exponents [rows], [ncols]
+    int mt, nt, chunks, nsplit, rows, ncols, sh;
+    double* C;
+  };
+  struct Unit {
+    int m, s, n0, n1;
+    __device__ Unit(const Job& J, int u) : m((u / J.nt) % J.mt), s(u / (J.nt * J.mt)), n0(u % J.nt), n1(n0 + 1) {}
+    __device__ const unsigned char* A(const Job& J, int) const { return J.A + (size_t)m * J.chunks * XA_BYTES; }
+    __device__ const unsigned char* B(const Job& J, int n) const { return J.B + (size_t)n * J.chunks * XB_BYTES; }
+    __device__ void range(const Job& J, int, int& c0, int& c1) const {
       const int L = (J.chunks + J.nsplit - 1) / J.nsplit;
       c0 = s * L;
       c1 = min(J.chunks, c0 + L);
     }
+  };
+  int row, part;
+  __device__ OpStore(const Job&, const Unit& U, int r, int p) : row(128 * U.m + r), part(p) {}
+  __device__ void tile(const Job& J, const Unit& U, int n, const long long (&y)[16]) {
+    if (row >= J.rows) return;
+    const int ea = J.ea[row], c0 = XN * n + 16 * part;
+    double* o = J.C + ((size_t)U.s * J.rows + row) * J.ncols + c0;
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+      if (c0 + e < J.ncols) o[e] = fix_to_double(y[e], ea + J.eb[c0 + e] - 62 + J.sh);
   }
+  __device__ void finish(const Job&, const Unit&, double (&)[3][128], bool) {}
 };
 
-template <bool DOT>
-__global__ void __launch_bounds__(X_THREADS, 1)
-    k_digit_gemm(const __grid_constant__ XJob J, int nunits, int* __restrict__ err, long long wait_cycles, int stall) {
-  extern __shared__ __align__(1024) unsigned char smraw[];
-  unsigned char* base = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-  XSmem& S = *reinterpret_cast<XSmem*>(base + X_ST * XST_BYTES);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) {
-    for (int s = 0; s < X_ST; ++s) {
-      mbar_init(&S.full[s], 1);
-      mbar_init(&S.empty[s], 1);
+// Self-energy: unit = (M tile, tau), all N tiles jt (32 columns J of Y1 beside the same J of Y2) over the
+// K chunks I <= J, dotted with M: D[row][tau].
+struct OpDot {
+  struct Job {
+    const unsigned char *A, *B;  // [M tile][chunk], [tau][N tile][chunk]
+    const int *ea, *eb;          // row exponents [rows], [tau][J]
+    int mt, nt, chunks, rows, sh;
+    const double2* M;            // M[k][J][p] of the job's first row
+    int np, ni, ntau, tau0, ntau_all, tgrp;
+    double* D;
+  };
+  struct Unit {
+    int m, b, n0, n1;
+    __device__ Unit(const Job& J, int u) : n0(0), n1(J.nt) {
+      // tau in groups of tgrp, inside a group the M tiles, inside those the group's tau: the blocks that run
+      // at one time share their W~ and M digits in L2
+      const int per = J.mt * J.tgrp, g = u / per, r = u % per, gt = min(J.tgrp, J.ntau - g * J.tgrp);
+      m = r / gt;
+      b = g * J.tgrp + r % gt;
     }
-    mbar_init(&S.done, 1);
-    for (int s = 0; s < XS_N; ++s) mbar_init(&S.lvl[s], X_EPI);
-    mbar_init(&S.fin, 1);
-    mbar_init(&S.never, 1);
-    S.abort_flag = 0;
-    S.no_dealloc = 0;
-    fence_mbar_init();
-  }
-  if (warp == X_EPI + 1) tmem_alloc(&S.tslot, 512);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tbase = S.tslot;
-
-  if (warp == X_EPI) {
-    // ------------------------------------------------------------ producer: one bulk copy per operand and chunk
-    if (lane == 0) {
-      int i = 0;  // running chunk: stage i % X_ST, its phase i / X_ST
-      bool live = true;
-      for (int u = blockIdx.x; u < nunits && live; u += gridDim.x) {
-        const XUnit<DOT> U(J, u);
-        for (int n = U.n0; n < U.n1 && live; ++n) {
-          int c0, c1;
-          U.range(J, n, c0, c1);
-          const unsigned char* a = J.A + (size_t)U.m * J.chunks * XA_BYTES;
-          const unsigned char* b = J.B + ((size_t)U.b * J.nt + n) * J.chunks * XB_BYTES;
-          for (int c = c0; c < c1; ++c, ++i) {
-            const int s = i % X_ST;
-            if (S.abort_flag ||
-                (i >= X_ST && !wait_bar(&S.empty[s], (i / X_ST + 1) & 1, &S.abort_flag, err, wait_cycles))) {
-              live = false;
-              break;
-            }
-            unsigned char* st = base + s * XST_BYTES;
-            mbar_arrive_expect_tx(&S.full[s], XST_BYTES);
-            bulk_g2s(st, a + (size_t)c * XA_BYTES, XA_BYTES, &S.full[s]);
-            bulk_g2s(st + XA_BYTES, b + (size_t)c * XB_BYTES, XB_BYTES, &S.full[s]);
-          }
-        }
-      }
-      // the copies of every issued chunk land before the block exits
-      for (int j = i > X_ST ? i - X_ST : 0; j < i; ++j)
-        if (!drain_bar(&S.full[j % X_ST], (j / X_ST) & 1)) S.no_dealloc = 1;
+    __device__ const unsigned char* A(const Job& J, int) const { return J.A + (size_t)m * J.chunks * XA_BYTES; }
+    __device__ const unsigned char* B(const Job& J, int n) const {
+      return J.B + ((size_t)b * J.nt + n) * J.chunks * XB_BYTES;
     }
-  } else if (warp == X_EPI + 1) {
-    // ------------------------------------------------------------ MMA issuer: the warp stays converged
-    const uint32_t id = idesc_f16(128, XN, false, false), lead = elect_one();
-    const uint32_t dh = (uint32_t)(sdesc_none(0, 0) >> 32);
-    const uint32_t a0 = (uint32_t)sdesc_none(smem_u32(base), 128 * 16);
-    const uint32_t b0 = (uint32_t)sdesc_none(smem_u32(base) + XA_BYTES, XN * 16);
-    int s = 0, ph = 0, blk = 0;  // stage and its phase of the running chunk
-    bool live = true;
-    if (stall && lead) wait_bar(&S.never, 0, &S.abort_flag, err, wait_cycles);  // injected stall: runs out
-    __syncwarp();
-    for (int u = blockIdx.x; u < nunits && live; u += gridDim.x) {
-      const XUnit<DOT> U(J, u);
-      for (int n = U.n0; n < U.n1 && live; ++n) {
-        int c0, c1;
-        U.range(J, n, c0, c1);
-        for (int cb = c0; cb < c1 && live; cb += X_BLK, ++blk) {
-          const int ce = min(cb + X_BLK, c1);
-          for (int c = cb; c < ce; ++c) {
-            live = __all_sync(0xffffffffu, wait_bar(&S.full[s], ph, &S.abort_flag, err, wait_cycles));
-            if (!live) break;
-            tc_fence_after();
-            const uint32_t a = a0 + s * (XST_BYTES >> 4), b = b0 + s * (XST_BYTES >> 4);
-            if (c == cb) {
-#pragma unroll
-              for (int l = 0; l < XS_N; ++l) {
-                // the previous block's level l has been read (its first MMA overwrites it)
-                if (blk > 0) {
-                  live = live && __all_sync(0xffffffffu, wait_bar(&S.lvl[l], (blk - 1) & 1, &S.abort_flag, err, wait_cycles));
-                  tc_fence_after();
-                }
-#pragma unroll
-                for (int x = 0; x <= l; ++x)
-                  mma_f16_warp(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, x > 0, lead);
-              }
-            } else {
-#pragma unroll
-              for (int l = 0; l < XS_N; ++l)
-#pragma unroll
-                for (int x = 0; x <= l; ++x)
-                  mma_f16_warp(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, 1, lead);
-            }
-            mma_commit_warp(&S.empty[s], lead);
-            if (++s == X_ST) {
-              s = 0;
-              ph ^= 1;
-            }
-            if (!live) break;
-          }
-          if (live) mma_commit_warp(&S.done, lead);
-        }
-      }
+    __device__ void range(const Job&, int n, int& c0, int& c1) const {
+      c0 = 0;
+      c1 = 4 * (n + 1);
     }
-    mma_commit_warp(&S.fin, lead);
-    if (!drain_bar(&S.fin, 0)) S.no_dealloc = 1;  // every MMA issued here has completed
-    __syncwarp();
-  } else {
-    // ------------------------------------------------------------ epilogue: 16 warps, 16 columns each
-    const int quad = warp & 3, part = warp >> 2;
-    const int r = 32 * quad + lane;
-    const uint32_t tw = tbase + ((uint32_t)(32 * quad) << 16) + 16 * part;
-    int blk = 0;
-    bool ok = true;  // uniform over the warp; a warp that gave up still takes part in the block barriers below
-    for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
-      const XUnit<DOT> U(J, u);
-      const int row = 128 * U.m + r;
-      const bool live = row < J.rows;
-      const int ea = live ? J.ea[row] : 0;
-      double dacc[4] = {0.0, 0.0, 0.0, 0.0};  // short chains: less rounding, and the FP64 latency overlaps
-      for (int n = U.n0; n < U.n1 && ok; ++n) {
-        int c0, c1;
-        U.range(J, n, c0, c1);
-        long long hi[16], lo[16];
+  };
+  int r, part, row;
+  double dacc[4] = {0.0, 0.0, 0.0, 0.0};  // short chains: less rounding, and the FP64 latency overlaps
+  __device__ OpDot(const Job&, const Unit& U, int r_, int p) : r(r_), part(p), row(128 * U.m + r_) {}
+  __device__ void tile(const Job& J, const Unit& U, int n, const long long (&y)[16]) {
+    if (row >= J.rows) return;
+    const int k = row / J.np, p = row - k * J.np, j0 = 32 * n + 16 * (part & 1);
+    const double2* Mr = J.M + ((size_t)k * J.ni + j0) * J.np + p;
+    const int* eb = J.eb + (size_t)(J.tau0 + U.b) * J.ni + j0;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) hi[e] = lo[e] = 0;
-        for (int cb = c0; cb < c1 && ok; cb += X_BLK, ++blk) {
-          ok = __all_sync(0xffffffffu, wait_bar(&S.done, blk & 1, &S.abort_flag, err, wait_cycles));
-          if (!ok) break;
-          tc_fence_after();
-#pragma unroll
-          for (int l = 0; l < XS_N; ++l) {
-            constexpr int kShift[XS_N] = {16, 8, 0, 24, 16, 8, 0};
-            float v[16];
-            tmem_ld16(tw + XN * l, v);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S.lvl[l]);  // the next block may overwrite this level
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const long long t = (long long)__float2int_rn(v[e]) * (1 << kShift[l]);
-              if (l < 3) hi[e] += t; else lo[e] += t;
-            }
-          }
-        }
-        if (!ok) break;
-        // element = (hi 2^32 + lo) 2^(ea + eb - 62) = y 2^(ea + eb - 62 + sh), |y| < 2^63
-        const int sh = J.sh;
-        if constexpr (DOT) {
-          if (live) {
-            const int k = row / J.np, p = row - k * J.np, j0 = 32 * n + 16 * (part & 1);
-            const double2* Mr = J.M + ((size_t)k * J.ni + j0) * J.np + p;
-            const int* eb = J.eb + (size_t)(J.tau0 + U.b) * J.ncols + j0;
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const double2 a = Mr[(size_t)e * J.np];
-              const long long y = (hi[e] << (32 - sh)) + (lo[e] >> sh);
-              dacc[e & 3] = fma(fix_to_double(y, eb[e] - 62 + sh), part >= 2 ? a.y : a.x, dacc[e & 3]);
-            }
-          }
-        } else if (live) {
-          double* o = J.C + ((size_t)U.s * J.rows + row) * J.ncols + XN * n + 16 * part;
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const int col = XN * n + 16 * part + e;
-            if (col < J.ncols)
-              o[e] = fix_to_double((hi[e] << (32 - sh)) + (lo[e] >> sh), ea + J.eb[col] - 62 + sh);
-          }
-        }
-      }
-      if constexpr (DOT) {
-        const double d = (dacc[0] + dacc[1]) + (dacc[2] + dacc[3]);
-        if (part) S.red[part - 1][r] = d;
-        asm volatile("bar.sync 1, %0;" ::"n"(X_EPI * 32) : "memory");
-        if (!part && live && ok)
-          J.D[(size_t)row * J.ntau_all + J.tau0 + U.b] =
-              ea == kBadExp ? __longlong_as_double(0x7FF8000000000000ll)
-                            : scalbn(2.0 * ((d + S.red[0][r]) + (S.red[1][r] + S.red[2][r])), ea);
-        asm volatile("bar.sync 1, %0;" ::"n"(X_EPI * 32) : "memory");
-      }
+    for (int e = 0; e < 16; ++e) {
+      const double2 a = Mr[(size_t)e * J.np];
+      dacc[e & 3] = fma(fix_to_double(y[e], eb[e] - 62 + J.sh), part >= 2 ? a.y : a.x, dacc[e & 3]);
     }
   }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == X_EPI + 1 && !S.no_dealloc) tmem_dealloc(tbase, 512);
-}
+  __device__ void finish(const Job& J, const Unit& U, double (&red)[3][128], bool ok) {
+    const double d = (dacc[0] + dacc[1]) + (dacc[2] + dacc[3]);
+    if (part) red[part - 1][r] = d;
+    asm volatile("bar.sync 1, %0;" ::"n"(X_EPI * 32) : "memory");
+    if (!part && ok && row < J.rows) {
+      const int ea = J.ea[row];
+      J.D[(size_t)row * J.ntau_all + J.tau0 + U.b] =
+          ea == kBadExp ? __longlong_as_double(0x7FF8000000000000ll)
+                        : scalbn(2.0 * ((d + red[0][r]) + (red[1][r] + red[2][r])), ea);
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(X_EPI * 32) : "memory");
+  }
+};
 
 // ------------------------------------------------------------------ polarization: preparation
 // FP64 pair weights w[tau][g], g = k np + p, of tau0 .. tau0 + nt - 1, and the largest high word of each tau
@@ -705,48 +405,6 @@ __global__ void k_xsig_sum(const double* __restrict__ D, const double* __restric
 // ------------------------------------------------------------------ host side
 constexpr size_t kXBudget = 2ull << 30;  // bytes of one operand's digits held at once
 
-// The context's digit workspace, grown on use. False (nothing launched, no error set) when it cannot
-// be had: no memory, or a capture in progress, where nothing may be allocated; the callers then run
-// the CUDA-core kernels, which need no workspace.
-bool x_workspace(gw_ctx* c, size_t need) {
-  if (need <= c->x_ws_bytes) return true;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
-  if (c->x_ws) cudaFree(c->x_ws);
-  c->x_ws = nullptr;
-  c->x_ws_bytes = 0;
-  if (cudaMalloc(&c->x_ws, need) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  c->x_ws_bytes = need;
-  return true;
-}
-
-// the sum of K products is below K 2^14 2^48 (1 + 2^-7): bits to drop so that it fits 63 bits
-int drop_bits(int64_t k) {
-  int b = 1;
-  while ((1ll << (b - 1)) < k) ++b;
-  return b;
-}
-
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-template <bool DOT>
-gw_status run_gemm(gw_ctx* c, const XJob& J, int nunits, const char* what) {
-  const size_t smem = 1024 + X_ST * XST_BYTES + sizeof(XSmem);
-  cudaFuncSetAttribute(k_digit_gemm<DOT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  if (sms < 1) sms = 148;
-  k_digit_gemm<DOT><<<std::min(nunits, sms), X_THREADS, smem, c->stream>>>(J, nunits, c->d_err, c->wait_cycles,
-                                                                          c->fault_stall);
-  return check_launch(c, what);
-}
-
 }  // namespace
 
 // P(tau) of one q in FP64. Returns GW_EUNSUPPORTED when the workspace cannot be had (see x_workspace).
@@ -777,8 +435,8 @@ gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P) {
                b_exp = align256(4 * ((size_t)ni + (size_t)ntau * ni)), b_y = align256(ych * nc),
                b_x = align256((size_t)mt * XA_BYTES * nc), b_c = align256(sizeof(double) * (size_t)nsplit * tg * ni * ni),
                b_e = align256(sizeof(double) * (size_t)ntau * ni * ni);
-  if (!x_workspace(c, b_w + b_max + b_exp + b_y + b_x + b_c + b_e)) return GW_EUNSUPPORTED;
-  char* q = (char*)c->x_ws;
+  if (!x_workspace(c, XW_POL, b_w + b_max + b_exp + b_y + b_x + b_c + b_e)) return GW_EUNSUPPORTED;
+  char* q = (char*)c->x_ws[XW_POL];
   double* w = (double*)q;
   uint32_t* wmax = (uint32_t*)(q += b_w);
   uint32_t *ymax = wmax + ntau, *xmax = ymax + ni;
@@ -812,7 +470,7 @@ gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P) {
                                                                                   tpt, t0 == 0, Yi, Xi);
       if ((st = check_launch(c, "exact pol digits")) != GW_OK) return st;
       const int sp = std::min(nsplit, (cn + X_BLK - 1) / X_BLK);
-      XJob J{};
+      OpStore::Job J{};
       J.A = Xi;
       J.B = Yi;
       J.ea = ex + (size_t)t0 * ni;
@@ -825,7 +483,7 @@ gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P) {
       J.ncols = ni;
       J.sh = drop_bits((int64_t)XK * ((cn + sp - 1) / sp));
       J.C = C;
-      if ((st = run_gemm<false>(c, J, J.mt * nt * sp, "exact pol gemm")) != GW_OK) return st;
+      if ((st = run_gemm<OpStore>(c, J, J.mt * nt * sp, "exact pol gemm")) != GW_OK) return st;
       const int64_t ne = (int64_t)tn * ni * ni;
       k_xsum<<<(unsigned)((ne + 255) / 256), 256, 0, c->stream>>>(C, ne, sp, c0 > 0, E + (size_t)t0 * ni * ni);
       if ((st = check_launch(c, "exact pol sum")) != GW_OK) return st;
@@ -846,8 +504,8 @@ gw_status launch_sigma_exact(gw_ctx* c, int iq, const double* G, const double* W
   const size_t b_ea = align256(sizeof(int) * (size_t)nk * np), b_ew = align256(sizeof(int) * (size_t)ntau * ni),
                b_a = align256((size_t)mtiles(kg) * ch * XA_BYTES), b_b = align256(b1 * tg),
                b_d = align256(sizeof(double) * (size_t)kg * np * ntau);
-  if (!x_workspace(c, b_ea + b_ew + b_a + b_b + b_d)) return GW_EUNSUPPORTED;
-  char* q = (char*)c->x_ws;
+  if (!x_workspace(c, XW_SIGMA, b_ea + b_ew + b_a + b_b + b_d)) return GW_EUNSUPPORTED;
+  char* q = (char*)c->x_ws[XW_SIGMA];
   int* ea = (int*)q;
   int* ew = (int*)(q += b_ea);
   unsigned char* Ai = (unsigned char*)(q += b_ew);
@@ -873,7 +531,7 @@ gw_status launch_sigma_exact(gw_ctx* c, int iq, const double* G, const double* W
                                                             ni, Bi);
         if ((st = check_launch(c, "exact sigma digits")) != GW_OK) return st;
       }
-      XJob J{};
+      OpDot::Job J{};
       J.A = Ai;
       J.B = Bi;
       J.ea = ea + (size_t)k0 * np;
@@ -882,7 +540,6 @@ gw_status launch_sigma_exact(gw_ctx* c, int iq, const double* G, const double* W
       J.nt = nt;
       J.chunks = ch;
       J.rows = rows;
-      J.ncols = ni;
       J.M = Mk;
       J.np = np;
       J.ni = ni;
@@ -892,7 +549,7 @@ gw_status launch_sigma_exact(gw_ctx* c, int iq, const double* G, const double* W
       J.sh = drop_bits(2 * ni);
       J.tgrp = 8;
       J.D = D;
-      if ((st = run_gemm<true>(c, J, J.mt * tn, "exact sigma gemm")) != GW_OK) return st;
+      if ((st = run_gemm<OpDot>(c, J, J.mt * tn, "exact sigma gemm")) != GW_OK) return st;
     }
     const int64_t ne = (int64_t)kn * c->nb * ntau;
     k_xsig_sum<<<(unsigned)((ne + 127) / 128), 128, 0, c->stream>>>(D, G, c->d_kmq + (size_t)iq * nk, k0, kn, c->nb, ntau,

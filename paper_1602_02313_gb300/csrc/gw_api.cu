@@ -273,129 +273,66 @@ gw_status launch_dyson(gw_ctx* c, const double* eps, const double* sigx, const d
 // Transforms: fixed FP64 matrices applied as batched matvecs.
 // ----------------------------------------------------------------------------
 // BOSE tau -> i nu: out[j][b] = sum_i T[j][i] in[i][b]  (complex T, complex data).
-// The arithmetic is a policy: FP64, or float-float (arith.cuh) on the FP32 pipes.
-// FP64 complex -> float-float, once per transform call.
-__global__ void k_to_ff(const double2* __restrict__ in, arith::Ff32::S* __restrict__ out, int64_t n) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) out[i] = arith::Ff32::from(in[i].x, in[i].y);
-}
-
-// ghat = (W_IJ + W_JI)/2 and hhat = (W_IJ - W_JI)/(2i) of a Hermitian-matrix function in
-// float-float, the same operations as k_bose_bwd's own (one pass over W instead of one per tau block).
-__global__ void k_to_ff_sym(const double2* __restrict__ W, int m, int64_t nf, arith::Ff32::S* __restrict__ G,
-                            arith::Ff32::S* __restrict__ H) {
-  using AR = arith::Ff32;
-  const int64_t mm = (int64_t)m * m;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= nf * mm) return;
-  const int64_t j = i / mm, e = i % mm;
-  const int I = (int)(e / m), J = (int)(e % m);
-  const double2 ad = W[i], bd = W[j * mm + (int64_t)J * m + I];
-  const AR::S a = AR::from(ad.x, ad.y), bv = AR::from(bd.x, bd.y);
-  G[i] = AR::half(AR::add(a, bv));
-  H[i] = AR::mul_mi(AR::half(AR::dif(a, bv)));
-}
-
-static gw_status grow_ws(gw_ctx* c, size_t need) {
-  if (need <= c->ff_ws_bytes) return GW_OK;
-  if (c->ff_ws) cudaFree(c->ff_ws);
-  c->ff_ws = nullptr;
-  c->ff_ws_bytes = 0;
-  if (cudaMalloc(&c->ff_ws, need) != cudaSuccess) {
-    cudaGetLastError();
-    return set_err(c, GW_ENOMEM, "transform workspace");
-  }
-  c->ff_ws_bytes = need;
-  return GW_OK;
-}
-
-// Input values in the policy's storage type (FP64 data as is; float-float data converted once
-// beforehand by k_to_ff, so that the FP64-pipe conversions are not repeated per frequency block).
-template <int JB, class AR>
-__global__ void k_bose_fwd(const double2* __restrict__ T, const typename AR::S* __restrict__ in,
-                           double2* __restrict__ out, int64_t batch, int ntau, int nf) {
-  // block (x, y, z): 128 batch elements x frequencies j0 .. j0 + JB - 1 (grid.y = ceil(nf / JB))
-  // of transform z
-  using S = typename AR::S;
+constexpr int BOSE_B = 8;  // frequencies (tau points) per block
+__global__ void k_bose_fwd(const double2* __restrict__ T, const double2* __restrict__ in, double2* __restrict__ out,
+                           int64_t batch, int ntau, int nf) {
+  // block (x, y, z): 128 batch elements x frequencies j0 .. j0 + 7 (grid.y = ceil(nf / 8)) of transform z
+  using AR = arith::Fp64;
   extern __shared__ __align__(16) unsigned char bfsm[];
-  S* sT = reinterpret_cast<S*>(bfsm);
+  double2* sT = reinterpret_cast<double2*>(bfsm);
   in += (size_t)blockIdx.z * ntau * batch;  // grid.z: consecutive transforms of one call
   out += (size_t)blockIdx.z * nf * batch;
-  const int j0 = blockIdx.y * JB, nj = min(JB, nf - j0);
-  for (int i = threadIdx.x; i < nj * ntau; i += blockDim.x) {
-    const double2 t = T[(size_t)j0 * ntau + i];
-    sT[i] = AR::from(t.x, t.y);
-  }
+  const int j0 = blockIdx.y * BOSE_B, nj = min(BOSE_B, nf - j0);
+  for (int i = threadIdx.x; i < nj * ntau; i += blockDim.x) sT[i] = T[(size_t)j0 * ntau + i];
   __syncthreads();
   const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (b >= batch) return;
-  typename AR::Acc acc[JB];
+  double2 acc[BOSE_B];
 #pragma unroll
-  for (int q = 0; q < JB; ++q) acc[q] = AR::azero();
+  for (int q = 0; q < BOSE_B; ++q) acc[q] = AR::azero();
   for (int i = 0; i < ntau; ++i) {
-    const S x = in[(size_t)i * batch + b];
+    const double2 x = in[(size_t)i * batch + b];
 #pragma unroll
-    for (int q = 0; q < JB; ++q)
+    for (int q = 0; q < BOSE_B; ++q)
       if (q < nj) AR::mac(acc[q], sT[q * ntau + i], x);
   }
 #pragma unroll
-  for (int q = 0; q < JB; ++q)
-    if (q < nj) out[(size_t)(j0 + q) * batch + b] = AR::to(AR::val(acc[q]));
+  for (int q = 0; q < BOSE_B; ++q)
+    if (q < nj) out[(size_t)(j0 + q) * batch + b] = acc[q];
 }
 
 // BOSE i nu -> tau of a Hermitian-matrix function W[j][I][J]:
 // ghat = (W_IJ + W_JI)/2 (transform of Re W(tau)), hhat = (W_IJ - W_JI)/(2i) (of Im W(tau));
 // Re W(tau_i) = sum_j A_ij Re ghat_j + B_ij Im ghat_j, Im W(tau_i) likewise with hhat.
-// PRE: ghat and hhat come precomputed in float-float (k_to_ff_sym) instead of from W.
-template <int IB, class AR, bool PRE>
-__global__ void k_bose_bwd(const double* __restrict__ Tb, const double2* __restrict__ W,
-                           const typename AR::S* __restrict__ Gh, const typename AR::S* __restrict__ Hh,
-                           double2* __restrict__ out, int m, int ntau, int nf) {
-  // block (x, y, z): 128 matrix elements x tau points i0 .. i0 + IB - 1 (grid.y = ceil(ntau / IB))
-  // of transform z
-  using S = typename AR::S;
-  using R = typename AR::R;
+__global__ void k_bose_bwd(const double* __restrict__ Tb, const double2* __restrict__ W, double2* __restrict__ out, int m,
+                           int ntau, int nf) {
+  // block (x, y, z): 128 matrix elements x tau points i0 .. i0 + 7 (grid.y = ceil(ntau / 8)) of transform z
+  using AR = arith::Fp64;
   extern __shared__ __align__(16) unsigned char bbsm[];
-  R* sTb = reinterpret_cast<R*>(bbsm);
-  {
-    const size_t zq = (size_t)blockIdx.z * m * m;
-    if (PRE) {
-      Gh += zq * nf;
-      Hh += zq * nf;
-    } else {
-      W += zq * nf;
-    }
-    out += zq * ntau;
-  }
-  const int i0 = blockIdx.y * IB, ni = min(IB, ntau - i0);
-  for (int i = threadIdx.x; i < ni * 2 * nf; i += blockDim.x) sTb[i] = AR::rfrom(Tb[(size_t)i0 * 2 * nf + i]);
+  double* sTb = reinterpret_cast<double*>(bbsm);
+  W += (size_t)blockIdx.z * m * m * nf;
+  out += (size_t)blockIdx.z * m * m * ntau;
+  const int i0 = blockIdx.y * BOSE_B, ni = min(BOSE_B, ntau - i0);
+  for (int i = threadIdx.x; i < ni * 2 * nf; i += blockDim.x) sTb[i] = Tb[(size_t)i0 * 2 * nf + i];
   __syncthreads();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t mm = (int64_t)m * m;
   if (e >= mm) return;
   const int I = (int)(e / m), J = (int)(e % m);
   const int64_t et = (int64_t)J * m + I;
-  typename AR::Acc acc[IB];  // re: Re W(tau), im: Im W(tau)
+  double2 acc[BOSE_B];  // re: Re W(tau), im: Im W(tau)
 #pragma unroll
-  for (int q = 0; q < IB; ++q) acc[q] = AR::azero();
+  for (int q = 0; q < BOSE_B; ++q) acc[q] = AR::azero();
   for (int j = 0; j < nf; ++j) {
-    S g, h;
-    if (PRE) {
-      g = Gh[(size_t)j * mm + e];
-      h = Hh[(size_t)j * mm + e];
-    } else {
-      const double2 ad = W[(size_t)j * mm + e], bd = W[(size_t)j * mm + et];
-      const S a = AR::from(ad.x, ad.y), bv = AR::from(bd.x, bd.y);
-      g = AR::half(AR::add(a, bv));
-      h = AR::mul_mi(AR::half(AR::dif(a, bv)));
-    }
+    const double2 a = W[(size_t)j * mm + e], b = W[(size_t)j * mm + et];
+    const double2 g = AR::half(AR::add(a, b)), h = AR::mul_mi(AR::half(AR::dif(a, b)));
 #pragma unroll
-    for (int q = 0; q < IB; ++q)
+    for (int q = 0; q < BOSE_B; ++q)
       if (q < ni) AR::rmac2(acc[q], sTb[q * 2 * nf + j], sTb[q * 2 * nf + nf + j], g, h);
   }
 #pragma unroll
-  for (int q = 0; q < IB; ++q)
-    if (q < ni) out[(size_t)(i0 + q) * mm + e] = AR::to(AR::val(acc[q]));
+  for (int q = 0; q < BOSE_B; ++q)
+    if (q < ni) out[(size_t)(i0 + q) * mm + e] = acc[q];
 }
 
 // FERMI tau -> i w of real rows: out[b][j] = sum_i T[j][i] in[b][i]; one thread per (b, j).
@@ -434,38 +371,20 @@ __global__ void k_fermi_bwd(const double* __restrict__ Tb, const double2* __rest
   out[e] = s;
 }
 
-// Float-float conversions of a multi-transform call go through the workspace in chunks of
-// transforms of at most this many bytes.
-constexpr size_t kFfWsCap = 2ull << 30;
-
 gw_status launch_transform(gw_ctx* c, int stat, int dir, int prec, int count, int64_t batch, const double* in,
                            double* out) {
   const int nt = c->ntau;
+  // GW_F32X2 (relative error ~1e-12): on the tensor cores, 1e-13 at most. GW_FP64 stays native: the digit
+  // products' 1.1e-13 on the 48-point grid (large cancelling entries) is above native FP64's 9.4e-15.
+  if (prec == GW_F32X2 && (dir == GW_TAU_TO_IW || dir == GW_IW_TO_TAU)) {
+    const gw_status st = launch_bose_exact(c, dir, count, batch, in, out);
+    if (st != GW_EUNSUPPORTED) return st;
+  }
   if (stat == GW_BOSE && dir == GW_TAU_TO_IW) {
     const int64_t blocks = (batch + 127) / 128;
-    if (prec == GW_F32X2) {
-      using S = arith::Ff32::S;
-      const int64_t per = (int64_t)nt * batch;  // inputs of one transform
-      const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(count, kFfWsCap / (sizeof(S) * per)));
-      gw_status st;
-      if ((st = grow_ws(c, sizeof(S) * per * chunk)) != GW_OK) return st;
-      const size_t sm = sizeof(S) * 16 * nt;
-      if (sm > 48 * 1024) cudaFuncSetAttribute(k_bose_fwd<16, arith::Ff32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      for (int z0 = 0; z0 < count; z0 += chunk) {
-        const int nz = std::min(chunk, count - z0);
-        const int64_t n = per * nz;
-        k_to_ff<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>((const double2*)in + per * z0, (S*)c->ff_ws, n);
-        if ((st = check_launch(c, "to_ff")) != GW_OK) return st;
-        k_bose_fwd<16, arith::Ff32><<<dim3((unsigned)blocks, (c->nnu + 15) / 16, nz), 128, sm, c->stream>>>(
-            (const double2*)c->d_Bfwd, (const S*)c->ff_ws, (double2*)out + (int64_t)c->nnu * batch * z0, batch, nt,
-            c->nnu);
-        if ((st = check_launch(c, "bose_fwd")) != GW_OK) return st;
-      }
-      return GW_OK;
-    }
-    const size_t sm = sizeof(double2) * 8 * nt;
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_bose_fwd<8, arith::Fp64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_bose_fwd<8, arith::Fp64><<<dim3((unsigned)blocks, (c->nnu + 7) / 8, count), 128, sm, c->stream>>>(
+    const size_t sm = sizeof(double2) * BOSE_B * nt;
+    if (sm > 48 * 1024) cudaFuncSetAttribute(k_bose_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_bose_fwd<<<dim3((unsigned)blocks, (c->nnu + BOSE_B - 1) / BOSE_B, count), 128, sm, c->stream>>>(
         (const double2*)c->d_Bfwd, (const double2*)in, (double2*)out, batch, nt, c->nnu);
     return check_launch(c, "bose_fwd");
   }
@@ -473,35 +392,10 @@ gw_status launch_transform(gw_ctx* c, int stat, int dir, int prec, int count, in
     const int m = (int)batch;
     const int64_t mm = (int64_t)m * m;
     const unsigned blocks = (unsigned)((mm + 127) / 128);
-    if (prec == GW_F32X2) {
-      using S = arith::Ff32::S;
-      const int64_t per = (int64_t)c->nnu * mm;  // inputs of one transform
-      const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(count, kFfWsCap / (2 * sizeof(S) * per)));
-      gw_status st;
-      if ((st = grow_ws(c, 2 * sizeof(S) * per * chunk)) != GW_OK) return st;
-      const size_t sm = sizeof(arith::Ff32::R) * 16 * 2 * c->nnu;
-      if (sm > 48 * 1024)
-        cudaFuncSetAttribute(k_bose_bwd<16, arith::Ff32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      for (int z0 = 0; z0 < count; z0 += chunk) {
-        const int nz = std::min(chunk, count - z0);
-        const int64_t n = per * nz;
-        S* Gh = (S*)c->ff_ws;
-        S* Hh = Gh + n;
-        // nz consecutive transforms are one [nz nnu][m][m] stack for the symmetrisation
-        k_to_ff_sym<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>((const double2*)in + per * z0, m,
-                                                                         (int64_t)c->nnu * nz, Gh, Hh);
-        if ((st = check_launch(c, "to_ff_sym")) != GW_OK) return st;
-        k_bose_bwd<16, arith::Ff32, true><<<dim3(blocks, (nt + 15) / 16, nz), 128, sm, c->stream>>>(
-            c->d_Bbwd, nullptr, Gh, Hh, (double2*)out + (int64_t)nt * mm * z0, m, nt, c->nnu);
-        if ((st = check_launch(c, "bose_bwd")) != GW_OK) return st;
-      }
-      return GW_OK;
-    }
-    const size_t sm = sizeof(double) * 8 * 2 * c->nnu;
-    if (sm > 48 * 1024)
-      cudaFuncSetAttribute(k_bose_bwd<8, arith::Fp64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_bose_bwd<8, arith::Fp64, false><<<dim3(blocks, (nt + 7) / 8, count), 128, sm, c->stream>>>(
-        c->d_Bbwd, (const double2*)in, nullptr, nullptr, (double2*)out, m, nt, c->nnu);
+    const size_t sm = sizeof(double) * BOSE_B * 2 * c->nnu;
+    if (sm > 48 * 1024) cudaFuncSetAttribute(k_bose_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_bose_bwd<<<dim3(blocks, (nt + BOSE_B - 1) / BOSE_B, count), 128, sm, c->stream>>>(
+        c->d_Bbwd, (const double2*)in, (double2*)out, m, nt, c->nnu);
     return check_launch(c, "bose_bwd");
   }
   // FERMI: count consecutive [batch][...] blocks are one batch of count * batch rows
@@ -759,6 +653,10 @@ gw_status gw_create(gw_ctx** out, const gw_grid* g, const gw_system* s, int devi
     return GW_ENOMEM;
   }
 
+  if ((st = bose_digits(c)) != GW_OK) {
+    gw_destroy(c);
+    return st;
+  }
   if (s->M) {
     c->d_M = s->M;
   } else {
@@ -818,12 +716,12 @@ gw_status gw_destroy(gw_ctx* c) {
   c->m_done.clear();
   if (c->m_stream) cudaStreamDestroy(c->m_stream);
   c->m_stream = nullptr;
-  if (c->ff_ws) cudaFree(c->ff_ws);
   if (c->d_tsys) cudaFree(c->d_tsys);
   if (c->d_dyt) cudaFree(c->d_dyt);
   if (c->d_dm) cudaFree(c->d_dm);
-  if (c->x_ws) cudaFree(c->x_ws);
-  c->ff_ws = nullptr;
+  for (void* p : c->x_ws)
+    if (p) cudaFree(p);
+  if (c->d_bdig) cudaFree(c->d_bdig);
   double* bufs[] = {c->d_sqrtv, c->d_v,       c->d_M_own, c->d_Bfwd,  c->d_Ffwd,  c->d_Fcont, c->d_Bbwd,
                     c->d_Fbwd,  c->d_Fbwd_beta, c->d_aug,   c->d_cpe_x, c->d_cpe_A, c->d_cpe_N, c->d_cpe_tab, c->d_cpe_b,
                     c->d_pade,  c->d_vm};

@@ -95,15 +95,13 @@ struct gw_ctx {
   double* d_cpe_x = nullptr;
   double* d_cpe_A = nullptr;    // real [2 ncont][ngrid]
   double* d_cpe_N = nullptr;    // real [ngrid][ngrid]: A^T A + lambda^2 I
-  double* d_cpe_tab = nullptr;
-  void* ff_ws = nullptr;        // float-float copies of a bosonic transform's input
+  double* d_cpe_tab = nullptr;  // real [1201][ngrid]: Re Phi_m on the QP scan grid
   void* d_tsys = nullptr;       // gw_screen_tau: two copies of the augmented system + increments
   size_t tsys_bytes = 0;
   void* d_dm = nullptr;         // gw_dyson_matrix: Sigma^c(i w), eigenpairs, augmented systems, remainders
   size_t dm_bytes = 0;
   void* d_dyt = nullptr;        // gw_dyson_tau: augmented systems of a chunk of states + the mesh
   size_t dyt_bytes = 0;
-  size_t ff_ws_bytes = 0;  // real [1201][ngrid]: Re Phi_m on the QP scan grid
   double* d_cpe_b = nullptr;    // [nprob][ngrid]
   size_t cpe_b_bytes = 0;
   int64_t cpe_nprob = 0;       // problems of the last GW_CPE call
@@ -114,8 +112,9 @@ struct gw_ctx {
   int64_t cpe_seed_nprob = 0;
   double* d_pade = nullptr;     // cplx [nprob][npade] coefficients
   size_t pade_bytes = 0;
-  void* x_ws = nullptr;         // FP64 contractions on the tensor cores: operand digits, partial sums
-  size_t x_ws_bytes = 0;
+  void* x_ws[5] = {};           // digit products on the tensor cores: operand digits, partial sums
+  size_t x_ws_bytes[5] = {};
+  void* d_bdig = nullptr;       // digits of the bosonic maps (digit_bose.cu)
   // tensor-core path
   gwi::MixedWork mw;
   int* d_err = nullptr;                     // error word of the bounded device waits (read by gw_sync)
@@ -153,6 +152,8 @@ gw_status launch_pol_fp64(gw_ctx* c, int iq, const double* G, double* P);
 // FP64 on the tensor cores (exact digit products); GW_EUNSUPPORTED when the digit workspace cannot be had
 gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P);
 gw_status launch_sigma_exact(gw_ctx* c, int iq, const double* G, const double* W, double* S);
+gw_status bose_digits(gw_ctx* c);  // at gw_create, after the transform matrices
+gw_status launch_bose_exact(gw_ctx* c, int dir, int count, int64_t batch, const double* in, double* out);
 gw_status launch_pol_mixed(gw_ctx* c, int iq, const double* G, int prec, double* P);
 gw_status launch_pol_many(int njobs, gw_ctx* const* ctxs, const int* iqs, const double* const* G, double* const* P);
 gw_status launch_transform(gw_ctx* c, int stat, int dir, int prec, int count, int64_t batch, const double* in,
