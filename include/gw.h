@@ -183,8 +183,9 @@ gw_status gw_tau_to_freq_many(gw_ctx* ctx, gw_stat stat, gw_dir dir, int count, 
  * passes) X = (1 - Pi)^-1 - 1 from a blocked in-place Gauss-Jordan inversion; the
  * elimination of [1 - Pi | Pi] (GW_FP64 only, any ni) serves gw_screen_static. No pivoting:
  * 1 - Pi has Hermitian part >= 1.
- * prec: GW_FP64 (native FP64), GW_F32X2 (float-float arithmetic; relative error ~1e-12
- * per element) or GW_F32 (FP32 arithmetic, blocked inversion only; relative error of the
+ * prec: GW_FP64 (native FP64), GW_F32X2 (pivot blocks in float-float, the updates as exact digit
+ * products on the tensor cores with up to 0.8 GiB of further workspace, or float-float throughout when
+ * that cannot be had; relative error ~1e-14 at ni = 256) or GW_F32 (FP32 arithmetic, blocked inversion only; relative error of the
  * order of sqrt(ni) 6e-8 cond(1 - Pi), ~1e-6 at ni = 256); else GW_EUNSUPPORTED.
  * P_iv, Wt_iv cplx [nqb][nnu][ni][ni]; info out (device) [nqb][nnu]: 0, or j+1 for a
  * zero pivot at elimination step j (that system's output is then undefined).

@@ -107,6 +107,27 @@ struct Ff32 {
     ffmac(a.ih, a.il, x.rh, x.rl, y.ih, y.il);
     ffmac(a.ih, a.il, x.ih, x.il, y.rh, y.rl);
   }
+  // (h, l) + (x y + z w), renormalised: the products first, so that one sum meets (h, l)
+  __device__ __forceinline__ static void ffmac2(float& h, float& l, float xh, float xl, float yh, float yl, float zh,
+                                                float zl, float wh, float wl) {
+    const float p = __fmul_rn(xh, yh), q = __fmul_rn(zh, wh);
+    float e = fmaf(xh, yh, -p), f = fmaf(zh, wh, -q);
+    e = fmaf(xh, yl, e);
+    f = fmaf(zh, wl, f);
+    e = fmaf(xl, yh, e);
+    f = fmaf(zl, wh, f);
+    const float s = p + q, v = s - p, r = (p - (s - v)) + (q - v);
+    const float t = h + s, u = t - h, g = (h - (t - u)) + (s - u);
+    h = t;
+    l = g + (l + (r + (e + f)));
+    renorm(h, l);
+  }
+  __device__ __forceinline__ static S fma2(S a, S x, S y) {  // a + x y
+    ffmac2(a.rh, a.rl, x.rh, x.rl, y.rh, y.rl, -x.ih, -x.il, y.ih, y.il);
+    ffmac2(a.ih, a.il, x.rh, x.rl, y.ih, y.il, x.ih, x.il, y.rh, y.rl);
+    return a;
+  }
+  __device__ __forceinline__ static S neg(S a) { return {-a.rh, -a.rl, -a.ih, -a.il}; }
   __device__ __forceinline__ static void renorm(float& h, float& l) {
     const float s = h + l;
     l = l - (s - h);
@@ -131,10 +152,22 @@ struct Ff32 {
     ffsub(b.ih, b.il, a.ih, a.il, r.ih, r.il);
     return r;
   }
-  __device__ static S inv(S v) {  // one reciprocal per pivot: in FP64
-    const double2 d = to(v);
-    const double2 r = cinv_d(d);
-    return from(r.x, r.y);
+  // 1 / v in FP64 without its division (~40 instructions of the FP64 pipe, 16 clocks each): v scaled by a
+  // power of two to about 1, 1 / |v|^2 by two Newton steps from the FP32 reciprocal
+  __device__ static S inv(S v) {
+    const uint32_t f = max(__float_as_uint(v.rh) & 0x7F800000u, __float_as_uint(v.ih) & 0x7F800000u) >> 23;
+    const float s = __uint_as_float((254u - min(max(f, 1u), 253u)) << 23);  // 2^(127 - f)
+    const double2 a = to(S{v.rh * s, v.rl * s, v.ih * s, v.il * s});
+    const double d = fma(a.x, a.x, a.y * a.y);
+    double q = (double)__frcp_rn((float)d);
+    q = fma(q, fma(-d, q, 1.0), q);
+    q = fma(q, fma(-d, q, 1.0), q);
+    S o = from(a.x * q, -a.y * q);
+    o.rh *= s;
+    o.rl *= s;
+    o.ih *= s;
+    o.il *= s;
+    return o;
   }
 };
 

@@ -337,7 +337,8 @@ gw_status launch_screen(gw_ctx* c, int iq0, int nqb, int prec, const double* P, 
   const bool blocked = c->ni % GJ_B == 0;
   if (prec == GW_F32X2) {
     if (!blocked) return set_err(c, GW_EUNSUPPORTED, "gw_screen: GW_F32X2 needs ni a multiple of 32");
-    return launch_inv<Ff32>(c, iq0, nsys, P, W, info, aug);
+    const gw_status st = launch_screen_digits(c, iq0, nqb, P, W, info, aug);
+    return st == GW_EUNSUPPORTED ? launch_inv<Ff32>(c, iq0, nsys, P, W, info, aug) : st;
   }
   if (prec == GW_F32) {
     if (!blocked) return set_err(c, GW_EUNSUPPORTED, "gw_screen: GW_F32 needs ni a multiple of 32");
