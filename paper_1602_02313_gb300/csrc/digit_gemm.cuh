@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(X_THREADS, 1)
       for (int j = i > X_ST ? i - X_ST : 0; j < i; ++j)
         if (!drain_bar(&S.full[j % X_ST], (j / X_ST) & 1)) S.no_dealloc = 1;
     }
+    __syncwarp();  // the warp meets the block barrier converged
   } else if (warp == X_EPI + 1) {
     // ------------------------------------------------------------ MMA issuer: the warp stays converged
     const uint32_t id = idesc_f16(128, XN, false, false), lead = elect_one();
@@ -252,29 +253,37 @@ __global__ void __launch_bounds__(X_THREADS, 1)
                   live = live && __all_sync(0xffffffffu, wait_bar(&S.lvl[l], (blk - 1) & 1, &S.abort_flag, err, wait_cycles));
                   tc_fence_after();
                 }
+                if (lead) {
 #pragma unroll
-                for (int x = 0; x <= l; ++x)
-                  mma_f16_warp(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, x > 0, lead);
+                  for (int x = 0; x <= l; ++x)
+                    mma_f16_lo(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, x > 0);
+                }
+                __syncwarp();
               }
             } else {
+              if (lead) {
 #pragma unroll
-              for (int l = 0; l < XS_N; ++l)
+                for (int l = 0; l < XS_N; ++l)
 #pragma unroll
-                for (int x = 0; x <= l; ++x)
-                  mma_f16_warp(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, 1, lead);
+                  for (int x = 0; x <= l; ++x)
+                    mma_f16_lo(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, 1);
+              }
             }
-            mma_commit_warp(&S.empty[s], lead);
+            if (lead) mma_commit(&S.empty[s]);
+            __syncwarp();
             if (++s == X_ST) {
               s = 0;
               ph ^= 1;
             }
             if (!live) break;
           }
-          if (live) mma_commit_warp(&S.done, lead);
+          if (live && lead) mma_commit(&S.done);
+          __syncwarp();
         }
       }
     }
-    mma_commit_warp(&S.fin, lead);
+    if (lead) mma_commit(&S.fin);
+    __syncwarp();
     if (!drain_bar(&S.fin, 0)) S.no_dealloc = 1;  // every MMA issued here has completed
     __syncwarp();
   } else {

@@ -38,6 +38,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// The same, suspended for up to about `ns` nanoseconds.
+__device__ __forceinline__ bool mbar_try_wait_for(uint64_t* bar, uint32_t parity, uint32_t ns) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
+      : "memory");
+  return ok != 0;
+}
 // Wait for the phase with the given parity to complete; gives up after the
 // budget, records kErrTimeout in *err and returns false.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err) {
@@ -64,7 +74,12 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
                                          long long budget) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
+  while (true) {
+    // The abort flag and the clock are looked at once in eight polls: every look is a load through the data
+    // pipe that the MMAs read their operands by (20 % of it, with eight warps waiting and a look per poll).
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i)
+      if (mbar_try_wait_for(bar, parity, 1000)) return true;
     if (*abort_flag) return false;
     if (clock64() - t0 > budget) {
       *abort_flag = 1;
@@ -72,7 +87,6 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
       return false;
     }
   }
-  return true;
 }
 
 // Wait for work this block has already issued (bulk copies into its shared memory, MMAs into its
@@ -196,30 +210,25 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
-// The forms for an issuer warp that runs converged: every lane computes the (uniform) operands and one
-// elected lane issues. In a lane == 0 branch the descriptors are per-thread values that cost a
-// register-to-uniform move each: measured 98 clocks per MMA of distinct descriptors, against the 48
-// that the operands of a 128 x 64 x 16 MMA take to read. desc_lo: low 32 bits of a descriptor
-// (address and leading offset), desc_hi the high 32, the same for A and B.
+// For an issuer warp that runs converged: the waits and the operands' arithmetic are the whole warp's (so
+// that they stay in uniform registers), and only the MMAs and commits stand in a branch of the one elected
+// lane. With the whole role in a lane == 0 branch the descriptors are per-thread values that cost a
+// register-to-uniform move each (measured 98 clocks per MMA of distinct descriptors, against the 48 that
+// the operands of a 128 x 64 x 16 MMA take to read). The branch is needed: uniform registers are the
+// warp's, so lanes that left a wait at different times must not both run through the issue code.
+// a_lo, b_lo: low 32 bits of the descriptors (address and leading offset), desc_hi: the high 32 of both.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t r;
   asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void mma_f16_warp(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                            uint32_t idesc, uint32_t accumulate, uint32_t lead) {
+__device__ __forceinline__ void mma_f16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                           uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n mov.b64 a, {%1, %3};\n mov.b64 b, {%2, %3};\n"
-      " setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n}" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit_warp(uint64_t* bar, uint32_t lead) {
-  asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
-      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(bar)),
-      "r"(lead)
+      "{\n .reg .pred p;\n .reg .b64 a, b;\n mov.b64 a, {%1, %3};\n mov.b64 b, {%2, %3};\n"
+      " setp.ne.b32 p, %5, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 

@@ -60,28 +60,37 @@ struct alignas(16) h8 {
 // --------------------------------------------------------------------------- polarization
 // E is covered by "strips": rows [128 i, 128 i + 128) x columns [c0, c0 + N), c0 = 0, 256, ...,
 // N <= 256 (the upper triangle of P in the complex form: c0 = 128 i, 128 i + 256, ...). A work
-// unit is (K segment, strip, tau). The unscaled
-// operand Y (rows of the strip's columns) is bulk-copied from YS, a pre-split,
+// unit is (K segment, strip, two tau) in the E form, (K segment, strip, tau) in the complex form: two
+// accumulators of N <= 256 columns fill the tensor memory in both, so that one copy of Y serves both
+// of them. A chunk is 32 pairs, its Re and its Im half 32 values of K each; a stage holds one half (E form)
+// or both (complex form): the operand Y (rows of the strip's columns), bulk-copied from YS, a pre-split,
 // pre-swizzled image of M[q]:
-//   YS[k][chunk][iblk][slice][128 rows x 128 B], row = [Re A (32 pairs) | Im A (32 pairs)],
-// slices hi, lo. The scaled operand X (rows of the strip) is built by the producer warps from the
-// same image. TMEM holds E (N columns), or Re P and Im P (N columns each).
+//   YS[k][chunk][iblk][Re, Im half][slice][128 rows x 64 B], slices hi, lo,
+// and the scaled operand X (rows of the strip), built by the producer warps from YS (complex form) or
+// from the FP32 image of the sums (E form)
+//   XF[k][chunk][iblk][half][128 rows][values 8 g + (0 .. 3), g = 0 .. 3, then 8 g + (4 .. 7)], halves
+//   re + im, im - re: a producer thread's two 16-byte reads of its 8 values are each beside its neighbours'.
 constexpr int kPolChunksPerSeg = 32;  // upper bound of the context's K chunks per segment
-constexpr int PT_THREADS = 288;                     // warps 0-7 produce / run the epilogue, warp 8 issues MMAs
-constexpr int P_XT = 16384;                         // one X slice: 128 rows x 128 B
-constexpr int P_STAGE_BYTES = 2 * P_XT + 2 * 256 * 128;  // X hi, lo (128 rows) + Y hi, lo (<= 256 rows)
+constexpr int PT_WARPS = 8;                         // warps 0-7 produce / run the epilogue
+constexpr int PT_THREADS = (PT_WARPS + 2) * 32;     // warp 8 issues MMAs, warp 9 the copies
+constexpr int P_SL = 128 * 64;                      // one X slice of a stage: 128 rows x 64 B
+constexpr int P_MAXST = 3;                          // stages: E form 3 x 64 KB, complex form 2 x 96 KB
+constexpr int P_SMEM = 192 * 1024;
 constexpr int P_TILE = 128 * 256;                   // floats of one unit's partial strip
 
 struct PolSmem {
-  uint64_t full[2], empty[2], done, never;  // never: nothing arrives on it (stall injection)
+  uint64_t fully[P_MAXST], fullx[P_MAXST], empty[P_MAXST], done;
+  uint64_t fin, never;                      // fin: all MMAs done; never: nothing arrives on it (stall injection)
   uint32_t tslot;
   int abort_flag;                           // any role gave up a wait
-  int abort_prod[2];                        // producer decision per chunk parity (uniform, see below)
   int no_dealloc;                           // issued work did not drain: keep TMEM, report only
 };
 
-__device__ __forceinline__ size_t ys_tile(int k, int c, int iblk, int sl, int cpk, int nib) {
-  return ((((size_t)k * cpk + c) * nib + iblk) * 2 + sl) * (size_t)(128 * 64);  // in halves
+__device__ __forceinline__ size_t ys_tile(int k, int c, int iblk, int half, int sl, int cpk, int nib) {
+  return (((((size_t)k * cpk + c) * nib + iblk) * 2 + half) * 2 + sl) * (size_t)(128 * 32);  // in halves
+}
+__device__ __forceinline__ size_t xf_tile(int k, int c, int iblk, int half, int cpk, int nib) {
+  return ((((size_t)k * cpk + c) * nib + iblk) * 2 + half) * (size_t)(128 * 32);  // in floats
 }
 
 // Pair weights of Eq. (irpol): wt[k][tau][p] = Q_ab(tau) = -G_b(k|tau) G_a(k-q|beta - tau),
@@ -99,9 +108,10 @@ __global__ void k_pol_weights(const double* __restrict__ G, const int* __restric
   wt[e] = w;
 }
 
-// M[q] -> YS (scaled by kScaleA, split into fp16 hi / lo). One thread per (k, I, 8 pairs).
-__global__ void k_split_y(const double2* __restrict__ Mq, int nk, int ni, int np, int cpk, int nib,
-                          __half* __restrict__ YS) {
+// M[q] -> YS (scaled by kScaleA, split into fp16 hi / lo) and, for the E form, XF (from the split values, so
+// that X is the product of a weight with exactly what Y holds). One thread per (k, I, 8 pairs).
+__global__ void k_split_y(const double2* __restrict__ Mq, int nk, int ni, int np, int cpk, int nib, int eform,
+                          __half* __restrict__ YS, float* __restrict__ XF) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t n = (int64_t)nk * ni * cpk * 4;
   if (e >= n) return;
@@ -119,44 +129,66 @@ __global__ void k_split_y(const double2* __restrict__ Mq, int nk, int ni, int np
     split2(cvt::d2f(v.y) * kScaleA, ih.v[q], il.v[q]);
   }
   const int iblk = I >> 7, r = I & 127;
-  __half* hi = YS + ys_tile(k, c, iblk, 0, cpk, nib);
-  __half* lo = YS + ys_tile(k, c, iblk, 1, cpk, nib);
-  *reinterpret_cast<h8*>(hi + sw128_off(r, 8 * g8) / 2) = rh;
-  *reinterpret_cast<h8*>(hi + sw128_off(r, 32 + 8 * g8) / 2) = ih;
-  *reinterpret_cast<h8*>(lo + sw128_off(r, 8 * g8) / 2) = rl;
-  *reinterpret_cast<h8*>(lo + sw128_off(r, 32 + 8 * g8) / 2) = il;
+  const uint32_t o = sw64_off(r, 8 * g8) / 2;
+  *reinterpret_cast<h8*>(YS + ys_tile(k, c, iblk, 0, 0, cpk, nib) + o) = rh;
+  *reinterpret_cast<h8*>(YS + ys_tile(k, c, iblk, 0, 1, cpk, nib) + o) = rl;
+  *reinterpret_cast<h8*>(YS + ys_tile(k, c, iblk, 1, 0, cpk, nib) + o) = ih;
+  *reinterpret_cast<h8*>(YS + ys_tile(k, c, iblk, 1, 1, cpk, nib) + o) = il;
+  if (!eform) return;
+  float x0[8], x1[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float re = __half2float(rh.v[q]) + __half2float(rl.v[q]), im = __half2float(ih.v[q]) + __half2float(il.v[q]);
+    x0[q] = re + im;
+    x1[q] = im - re;
+  }
+  float4* f0 = reinterpret_cast<float4*>(XF + xf_tile(k, c, iblk, 0, cpk, nib) + r * 32) + g8;
+  float4* f1 = reinterpret_cast<float4*>(XF + xf_tile(k, c, iblk, 1, cpk, nib) + r * 32) + g8;
+  f0[0] = make_float4(x0[0], x0[1], x0[2], x0[3]);
+  f0[4] = make_float4(x0[4], x0[5], x0[6], x0[7]);
+  f1[0] = make_float4(x1[0], x1[1], x1[2], x1[3]);
+  f1[4] = make_float4(x1[4], x1[5], x1[6], x1[7]);
 }
 
 // One polarization job: the operands of one (context, q) and where its partials go.
 struct PolJob {
   const __half* YS;
-  const float* wt;
+  const float *XF, *wt;
   float* part;
   const int4* strips;
   int nk, ni, ntau, cpk, npw, nstrips, nseg, seg0;
-  int eform;  // 1: strips of E (one accumulator); 0: strips of the Hermitian half (Re P, Im P)
-  int units;  // K segments x strips x tau of this job (this launch's segments)
+  int eform;  // 1: strips of E, two tau per unit; 0: strips of the Hermitian half (Re P, Im P), one tau
+  int units;  // K segments x strips x (tau / 2 or tau) of this job (this launch's segments)
 };
 
-// Barrier phases of a block that runs several work units one after another: the chunk counter
-// runs on across units (stage = chunk & 1, phase of that stage = chunk >> 1), and the MMA thread
-// commits `done` once per unit.
+// Barrier phases of a block that runs several work units one after another, kept by every role for
+// itself: bit s of `ph` is the phase of stage s's next use; the MMA warp commits `done` once per unit.
 struct PolPhase {
-  int cbase = 0;   // chunks of the units already run by this block
-  int units = 0;   // units already run (commits of `done`)
-  int last0 = -1;  // (thread 0) last chunk whose copies went to stage 0 / 1
-  int last1 = -1;
+  uint32_t ph = 0;
+  int s = 0;      // next stage (0 at the start of a unit that may change the number of stages)
+  int units = 0;  // units already run (commits of `done`)
+  uint32_t used = 0, uph = 0;  // copy thread: stages ever filled, and the phase of each one's last copy
 };
 
-// One work unit u of job J = (K segment, 128 x N strip, tau): the producer warps build
-// X = [w (Re A + Im A) | w (Im A - Re A)] (E form) or [w Re A | w Im A] (complex form) and bring Y
-// by bulk copy, one thread issues the MMAs, the producer warps then move the FP32 partial strip out
-// of TMEM. A wait that runs out raises S.abort_flag.
+__device__ __forceinline__ void pol_next(PolPhase& ph, int nst) {
+  ph.ph ^= 1u << ph.s;
+  ph.s = ph.s + 1 == nst ? 0 : ph.s + 1;
+}
+
+// One work unit u of job J: the copy warp brings Y, the producer warps build X, the MMA warp issues the
+// products into two accumulators, the producer warps then move the FP32 partial strips out of TMEM. A
+// wait that runs out raises S.abort_flag. What bounds it is the data pipe of shared memory and L1 (ncu:
+// 51 % MMA operands, 53 % producers and copies), at 73 % of the tensor pipe's cycles: in the E form at
+// N = 256 the 24 MMAs of a chunk and two tau read 2304 clocks' worth (128 bytes a clock) and take 3072.
+// One tau per unit brought Y twice as often (62 bytes of L2 per clock and SM at full rate) and converted
+// the halves of Y again per tau. Measured per q at Nk 64, Nb 64, NI 256, 48 tau: 7.85 -> 5.53 ms, the same
+// bits; complex form (NI 384, Nb 96, Nk 8, 48 tau) 4.97 -> 4.85 ms. XF through a shared-memory ring instead
+// of from L2 by the producers: 5.96 ms; both halves of the complex form in stages of their own: 5.10 ms.
 __device__ __forceinline__ void pol_unit(const PolJob& J, int u, PolSmem& S, unsigned char* base, uint32_t tbase,
-                                         int tid, int warp, int lane, PolPhase& ph, int* err, long long wait_cycles,
-                                         int stall) {
+                                         int warp, int lane, PolPhase& ph, int* err, long long wait_cycles, int stall) {
   const int ntau = J.ntau, nstrips = J.nstrips, cpk = J.cpk, npw = J.npw;
-  const int it = u % ntau, strip = (u / ntau) % nstrips, seg = J.seg0 + u / (ntau * nstrips);
+  const int nt = J.eform ? 2 : 1, nt_u = ntau / nt;  // tau per unit (ntau is even)
+  const int it = nt * (u % nt_u), strip = (u / nt_u) % nstrips, seg = J.seg0 + u / (nt_u * nstrips);
   const int4 sd = J.strips[strip];  // (row block, c0, N, -)
   const int xb = sd.x, c0 = sd.y, N = sd.z;
   const int nib = (J.ni + 127) / 128;
@@ -164,141 +196,230 @@ __device__ __forceinline__ void pol_unit(const PolJob& J, int u, PolSmem& S, uns
   const int L = (total + J.nseg - 1) / J.nseg;
   const int g0 = seg * L, g1 = min(total, g0 + L);
   const int nchunk = max(0, g1 - g0);
-  const uint32_t ybytes_slice = (uint32_t)N * 128;
-  const __half* YS = J.YS;
-  const float* wt = J.wt;
+  // stages of hps halves; in a stage X of its halves (each [tau][hi, lo]), then Y of its halves ([hi, lo])
+  const int hps = J.eform ? 1 : 2, nst = J.eform ? 3 : 2, stage = P_SMEM / nst, xhalf = nt * 2 * P_SL, ybase = hps * xhalf;
+  const uint32_t yslice = (uint32_t)N * 64;
 
-  if (warp < 8) {
+  if (warp < PT_WARPS) {
     // ------------------------------------------------------------ producers
-    // X for the strip's 128 rows: 512 items of (row, 8 pairs), two per thread. Within a
-    // warp, the 8 lanes of each quarter take rows r and r + 4 (r < 4 of an 8-row group), so
-    // their 16-byte stores land in 8 distinct bank groups of the 128-byte swizzle. The next
-    // chunk's operands and weights are loaded while the current chunk is written.
-    struct Item {
-      h8 rh, rl, ih, il;
-      float4 w0, w1;
+    // X of a half: 128 rows x 32 values (4 groups of 8) for each tau; a thread takes group lane & 3 of rows
+    // 8 warp + lane / 4 and + 64 (the 8 lanes of a quarter warp store two whole 64-byte rows). The next
+    // chunk's weights and the next half's values are loaded while the current ones are converted.
+    const int g = lane & 3, r0 = 8 * warp + (lane >> 2);
+    const uint32_t o0 = sw64_off(r0, 8 * g), o1 = sw64_off(r0 + 64, 8 * g);
+    struct Val {
+      uint4 a[2][2];  // [row]: 8 floats (E form), or 8 hi and 8 lo halves
     };
-    int ir[2], ig[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int item = tid + 256 * j, ln = item & 31;
-      ir[j] = 8 * (item >> 5) + ((ln & 7) >> 2) * 4 + (ln >> 3);
-      ig[j] = ln & 3;
-    }
-    auto fetch = [&](int i, Item (&it2)[2]) {
-      const int g = g0 + i, k = g / cpk, c = g % cpk;
-      const __half* xh = YS + ys_tile(k, c, xb, 0, cpk, nib);
-      const __half* xl = YS + ys_tile(k, c, xb, 1, cpk, nib);
-      const float* wrow = wt + ((size_t)k * ntau + it) * npw + c * 32;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const uint32_t oRe = sw128_off(ir[j], 8 * ig[j]), oIm = sw128_off(ir[j], 32 + 8 * ig[j]);
-        it2[j].rh = *reinterpret_cast<const h8*>(xh + oRe / 2);
-        it2[j].rl = *reinterpret_cast<const h8*>(xl + oRe / 2);
-        it2[j].ih = *reinterpret_cast<const h8*>(xh + oIm / 2);
-        it2[j].il = *reinterpret_cast<const h8*>(xl + oIm / 2);
-        it2[j].w0 = __ldg(reinterpret_cast<const float4*>(wrow + 8 * ig[j]));
-        it2[j].w1 = __ldg(reinterpret_cast<const float4*>(wrow + 8 * ig[j]) + 1);
-      }
+    struct Wgt {
+      float4 w[2][2];  // [tau][4 weights]
     };
-    Item cur[2], nxt[2];
-    if (nchunk > 0) fetch(0, cur);
-    for (int i = 0; i < nchunk; ++i) {
-      const int ic = ph.cbase + i, s = ic & 1;
-      // All 256 producer threads take the same go / stop decision for chunk ic (their flag slot is
-      // written only before this barrier, and slot ic & 1 is not written again before every thread
-      // has read it), so every chunk whose copies are issued gets all its arrivals and its full
-      // barrier completes once the bytes land: the drain can wait for it.
-      if (ic >= 2 && !wait_bar(&S.empty[s], ((ic >> 1) + 1) & 1, &S.abort_flag, err, wait_cycles)) S.abort_prod[s] = 1;
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (S.abort_prod[s]) break;
-      unsigned char* st = base + s * P_STAGE_BYTES;
-      if (tid == 0) {
-        // Y: rows [c0, c0 + N) = whole or leading parts of 128-row blocks, hi and lo slices
-        const int g = g0 + i, k = g / cpk, c = g % cpk;
-        if (s) ph.last1 = ic; else ph.last0 = ic;
-        mbar_arrive_expect_tx(&S.full[s], 2 * ybytes_slice);
-        for (int r0 = 0; r0 < N; r0 += 128) {
-          const int rows = min(128, N - r0);
-          const int yb = (c0 + r0) >> 7;
-          for (int sl = 0; sl < 2; ++sl)
-            bulk_g2s(st + 2 * P_XT + sl * ybytes_slice + r0 * 128, YS + ys_tile(k, c, yb, sl, cpk, nib),
-                     (uint32_t)rows * 128, &S.full[s]);
+    auto fetch = [&](int i, int half, Val& v) {
+      const int gg = g0 + i, k = gg / cpk, c = gg - k * cpk;
+      if (J.eform) {
+        const float* x = J.XF + xf_tile(k, c, xb, half, cpk, nib) + r0 * 32 + 4 * g;
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) v.a[j][q] = __ldg(reinterpret_cast<const uint4*>(x + j * 64 * 32) + 4 * q);
+      } else {
+        const __half* x = J.YS + ys_tile(k, c, xb, half, 0, cpk, nib);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          v.a[0][q] = __ldg(reinterpret_cast<const uint4*>(x + q * 128 * 32 + o0 / 2));
+          v.a[1][q] = __ldg(reinterpret_cast<const uint4*>(x + q * 128 * 32 + o1 / 2));
         }
       }
-      if (i + 1 < nchunk) fetch(i + 1, nxt);
+    };
+    auto weights = [&](int i, Wgt& w) {
+      const int gg = g0 + i, k = gg / cpk, c = gg - k * cpk;
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const uint32_t oRe = sw128_off(ir[j], 8 * ig[j]), oIm = sw128_off(ir[j], 32 + 8 * ig[j]);
-        const float wv[8] = {cur[j].w0.x, cur[j].w0.y, cur[j].w0.z, cur[j].w0.w,
-                             cur[j].w1.x, cur[j].w1.y, cur[j].w1.z, cur[j].w1.w};
-        h8 orh, orl, oih, oil;
+      for (int t = 0; t < 2; ++t) {
+        if (t == nt) break;
+        const float* x = J.wt + ((size_t)k * ntau + it + t) * npw + c * 32 + 8 * g;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float re = __half2float(cur[j].rh.v[e]) + __half2float(cur[j].rl.v[e]);
-          const float im = __half2float(cur[j].ih.v[e]) + __half2float(cur[j].il.v[e]);
-          split2(wv[e] * (J.eform ? re + im : re), orh.v[e], orl.v[e]);
-          split2(wv[e] * (J.eform ? im - re : im), oih.v[e], oil.v[e]);
-        }
-        *reinterpret_cast<h8*>(st + oRe) = orh;
-        *reinterpret_cast<h8*>(st + oIm) = oih;
-        *reinterpret_cast<h8*>(st + P_XT + oRe) = orl;
-        *reinterpret_cast<h8*>(st + P_XT + oIm) = oil;
+        for (int q = 0; q < 2; ++q) w.w[t][q] = __ldg(reinterpret_cast<const float4*>(x) + q);
       }
-      fence_proxy_async_smem();
-      mbar_arrive(&S.full[s]);
-#pragma unroll
-      for (int j = 0; j < 2; ++j) cur[j] = nxt[j];
+    };
+    Val cur, nxt;
+    Wgt w, wn;
+    bool ok = nchunk > 0;
+    if (ok) {
+      fetch(0, 0, cur);
+      weights(0, w);
     }
-  } else if (lane == 0) {
-    // ------------------------------------------------------------ MMA issuer
+    for (int i = 0; i < nchunk && ok; ++i) {
+      if (i + 1 < nchunk) weights(i + 1, wn);
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        if (half == 0) fetch(i, 1, nxt);
+        else if (i + 1 < nchunk) fetch(i + 1, 0, nxt);
+        const int s = ph.s;
+        if (half == 0 || hps == 1) {
+          ok = __all_sync(0xffffffffu, wait_bar(&S.empty[s], ((ph.ph >> s) & 1) ^ 1, &S.abort_flag, err, wait_cycles));
+          if (!ok) break;
+        }
+        float v[2][8];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t r[8] = {cur.a[j][0].x, cur.a[j][0].y, cur.a[j][0].z, cur.a[j][0].w,
+                                 cur.a[j][1].x, cur.a[j][1].y, cur.a[j][1].z, cur.a[j][1].w};
+          if (J.eform) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[j][e] = __uint_as_float(r[e]);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&r[e]));
+              const float2 l = __half22float2(*reinterpret_cast<const __half2*>(&r[4 + e]));
+              v[j][2 * e] = h.x + l.x;
+              v[j][2 * e + 1] = h.y + l.y;
+            }
+          }
+        }
+        unsigned char* st = base + s * stage + (hps == 1 ? 0 : half * xhalf);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          if (t == nt) break;
+          const float wv[8] = {w.w[t][0].x, w.w[t][0].y, w.w[t][0].z, w.w[t][0].w,
+                               w.w[t][1].x, w.w[t][1].y, w.w[t][1].z, w.w[t][1].w};
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float p0 = wv[2 * e] * v[j][2 * e], p1 = wv[2 * e + 1] * v[j][2 * e + 1];
+              const __half2 h = __floats2half2_rn(p0, p1);
+              const float2 f = __half22float2(h);
+              const __half2 l = __floats2half2_rn(p0 - f.x, p1 - f.y);
+              hi[e] = *reinterpret_cast<const uint32_t*>(&h);
+              lo[e] = *reinterpret_cast<const uint32_t*>(&l);
+            }
+            unsigned char* x = st + t * 2 * P_SL + (j ? o1 : o0);
+            *reinterpret_cast<uint4*>(x) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(x + P_SL) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          }
+        }
+        cur = nxt;
+        if (half == 1 || hps == 1) {
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&S.fullx[s]);
+          pol_next(ph, nst);
+        }
+      }
+      w = wn;
+    }
+  } else if (warp == PT_WARPS) {
+    // ------------------------------------------------------------ MMA issuer: the warp stays converged
+    const uint32_t lead = elect_one();
     const uint32_t id = idesc_f16(128, N, false, false), idn = idesc_f16(128, N, false, true);
-    const uint32_t dim = tbase + N;  // Im P (complex form)
-    if (stall && ph.units == 0) wait_bar(&S.never, 0, &S.abort_flag, err, wait_cycles);  // injected stall
-    for (int i = 0; i < nchunk; ++i) {
-      const int ic = ph.cbase + i, s = ic & 1;
-      if (S.abort_flag || !wait_bar(&S.full[s], (ic >> 1) & 1, &S.abort_flag, err, wait_cycles)) break;
+    const uint32_t dh = (uint32_t)(sdesc_sw64(0) >> 32), d0 = (uint32_t)sdesc_sw64(smem_u32(base));
+    if (stall && ph.units == 0 && lead) wait_bar(&S.never, 0, &S.abort_flag, err, wait_cycles);  // injected stall
+    __syncwarp();
+    bool live = true;
+    auto full = [&]() {  // half of the lanes wait for Y, half for X
+      uint64_t* bar = lane & 1 ? &S.fullx[ph.s] : &S.fully[ph.s];
+      live = live && __all_sync(0xffffffffu, !S.abort_flag && wait_bar(bar, (ph.ph >> ph.s) & 1, &S.abort_flag, err, wait_cycles));
       tc_fence_after();
-      const uint32_t st = smem_u32(base + s * P_STAGE_BYTES);
-      const uint32_t xh = st, xl = st + P_XT, yh = st + 2 * P_XT, yl = yh + ybytes_slice;
+    };
+    for (int i = 0; i < nchunk && live; ++i) {
+      if (J.eform) {
+        // E of two tau: Re half (K steps 0, 1), then Im half (2, 3), hi hi + hi lo + lo hi each
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        const uint32_t acc = (i > 0 || ks > 0) ? 1u : 0u;
-        const uint32_t bo = 32 * ks;
-        mma_f16(tbase, sdesc_sw128(xh + bo), sdesc_sw128(yh + bo), id, acc);
-        mma_f16(tbase, sdesc_sw128(xh + bo), sdesc_sw128(yl + bo), id, 1);
-        mma_f16(tbase, sdesc_sw128(xl + bo), sdesc_sw128(yh + bo), id, 1);
-        if (!J.eform) {
-          // Im P = [w Im A | -w Re A] . [Re A | Im A]: other K half of X, negated for the second half
-          const uint32_t ao = 32 * ((ks + 2) & 3);
-          const uint32_t idx = ks < 2 ? id : idn;
-          mma_f16(dim, sdesc_sw128(xh + ao), sdesc_sw128(yh + bo), idx, acc);
-          mma_f16(dim, sdesc_sw128(xh + ao), sdesc_sw128(yl + bo), idx, 1);
-          mma_f16(dim, sdesc_sw128(xl + ao), sdesc_sw128(yh + bo), idx, 1);
+        for (int half = 0; half < 2; ++half) {
+          full();
+          if (!live) break;
+          const uint32_t x = d0 + ph.s * (stage >> 4), yh = x + (ybase >> 4), yl = yh + (yslice >> 4);
+          if (lead) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const uint32_t d = tbase + 256 * t, xh = x + t * (2 * P_SL >> 4), xl = xh + (P_SL >> 4);
+#pragma unroll
+              for (int ks = 0; ks < 2; ++ks) {
+                const uint32_t acc = (i > 0 || half > 0 || ks > 0) ? 1u : 0u;
+                mma_f16_lo(d, xh + 2 * ks, yh + 2 * ks, dh, id, acc);
+                mma_f16_lo(d, xh + 2 * ks, yl + 2 * ks, dh, id, 1);
+                mma_f16_lo(d, xl + 2 * ks, yh + 2 * ks, dh, id, 1);
+              }
+            }
+            mma_commit(&S.empty[ph.s]);
+          }
+          __syncwarp();
+          pol_next(ph, nst);
         }
+      } else {
+        // Re P = X Y^T and Im P = [w Im A | -w Re A] . [Re A | Im A] (the other half of X, negated for the
+        // second K half)
+        full();
+        if (!live) break;
+        const uint32_t xr = d0 + ph.s * (stage >> 4), yr = xr + (ybase >> 4);
+        if (lead) {
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) {
+            const uint32_t o = 2 * (ks & 1), h = ks >> 1;
+            const uint32_t x = xr + h * (2 * P_SL >> 4) + o, xi = xr + (h ^ 1) * (2 * P_SL >> 4) + o;
+            const uint32_t yh = yr + h * (2 * yslice >> 4) + o, yl = yh + (yslice >> 4);
+            const uint32_t acc = (i > 0 || ks > 0) ? 1u : 0u, idx = h ? idn : id;
+            mma_f16_lo(tbase, x, yh, dh, id, acc);
+            mma_f16_lo(tbase, x, yl, dh, id, 1);
+            mma_f16_lo(tbase, x + (P_SL >> 4), yh, dh, id, 1);
+            mma_f16_lo(tbase + 256, xi, yh, dh, idx, acc);
+            mma_f16_lo(tbase + 256, xi, yl, dh, idx, 1);
+            mma_f16_lo(tbase + 256, xi + (P_SL >> 4), yh, dh, idx, 1);
+          }
+          mma_commit(&S.empty[ph.s]);
+        }
+        __syncwarp();
+        pol_next(ph, nst);
       }
-      mma_commit(&S.empty[s]);
     }
-    mma_commit(&S.done);
+    if (lead) mma_commit(&S.done);
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ copies of Y, by one lane
+    // rows [c0, c0 + N) = whole or leading parts of 128-row blocks, hi and lo slices
+    for (int i = 0; i < (lane == 0 ? nchunk : 0); ++i) {
+      const int gg = g0 + i, k = gg / cpk, c = gg - k * cpk;
+      for (int half = 0; half < 2; ++half) {
+        const int s0 = ph.s;
+        if (half == 0 || hps == 1) {
+          if (S.abort_flag || !wait_bar(&S.empty[s0], ((ph.ph >> s0) & 1) ^ 1, &S.abort_flag, err, wait_cycles)) {
+            i = nchunk;
+            break;
+          }
+          mbar_arrive_expect_tx(&S.fully[s0], hps * 2 * yslice);
+          ph.used |= 1u << s0;
+          ph.uph = (ph.uph & ~(1u << s0)) | (ph.ph & (1u << s0));
+        }
+        unsigned char* y = base + s0 * stage + ybase + (hps == 1 ? 0 : half * 2 * yslice);
+        for (int rr = 0; rr < N; rr += 128)
+          for (int sl = 0; sl < 2; ++sl)
+            bulk_g2s(y + sl * yslice + rr * 64, J.YS + ys_tile(k, c, (c0 + rr) >> 7, half, sl, cpk, nib),
+                     (uint32_t)min(128, N - rr) * 64, &S.fully[s0]);
+        if (half == 1 || hps == 1) pol_next(ph, nst);
+      }
+    }
+    __syncwarp();  // the queue's block barriers count whole warps: its other lanes must not meet them early
   }
 
-  // ------------------------------------------------------------ epilogue: FP32 partial strip (8 warps)
-  // The next unit's MMAs overwrite TMEM only after these threads have armed its first chunk.
-  if (warp < 8) {
-    const bool ok = nchunk > 0 && wait_bar(&S.done, ph.units & 1, &S.abort_flag, err, wait_cycles) && !S.abort_flag;
+  // ------------------------------------------------------------ epilogue: FP32 partial strips (8 warps)
+  // The next unit's MMAs overwrite TMEM only after these warps have built its first stage.
+  if (warp < PT_WARPS) {
+    const bool ok = nchunk > 0 &&
+                    __all_sync(0xffffffffu, wait_bar(&S.done, ph.units & 1, &S.abort_flag, err, wait_cycles) && !S.abort_flag);
     tc_fence_after();
     const int quad = warp & 3, half = warp >> 2;
     const int row = 32 * quad + lane;
-    const int nacc = J.eform ? 1 : 2;
-    float* out = J.part + (size_t)u * nacc * P_TILE + (size_t)row * 256;
+    // partial of unit u: [tau] (E form, two tau of this unit) or [Re, Im]: two tiles either way
+    float* out = J.part + (size_t)u * 2 * P_TILE + (size_t)row * 256;
     const int nb16 = N / 16;
     const int ab = 4 * xb + quad;  // the 32-row block of this warp's rows
-    for (int acc = 0; acc < nacc; ++acc) {
+    for (int acc = 0; acc < 2; ++acc) {
       for (int bk = half; bk < nb16; bk += 2) {
         if (!J.eform && ((c0 + 16 * bk) >> 5) < ab) continue;  // below the diagonal: never read back
         float v[16];
         if (ok) {
-          tmem_ld16(tbase + ((uint32_t)(32 * quad) << 16) + acc * N + 16 * bk, v);
+          tmem_ld16(tbase + ((uint32_t)(32 * quad) << 16) + 256 * acc + 16 * bk, v);
         } else {
 #pragma unroll
           for (int e = 0; e < 16; ++e) v[e] = 0.f;
@@ -310,67 +431,60 @@ __device__ __forceinline__ void pol_unit(const PolJob& J, int u, PolSmem& S, uns
     }
     tc_fence_before();
   }
-  ph.cbase += nchunk;
   ph.units += 1;
 }
 
 __device__ __forceinline__ void pol_block_init(PolSmem& S, int tid, int warp) {
   if (tid == 0) {
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&S.full[s], 257);
+    for (int s = 0; s < P_MAXST; ++s) {
+      mbar_init(&S.fully[s], 1);
+      mbar_init(&S.fullx[s], PT_WARPS);
       mbar_init(&S.empty[s], 1);
     }
     mbar_init(&S.done, 1);
+    mbar_init(&S.fin, 1);
     mbar_init(&S.never, 1);
     S.abort_flag = 0;
-    S.abort_prod[0] = S.abort_prod[1] = 0;
     S.no_dealloc = 0;
     fence_mbar_init();
   }
-  if (warp == 8) tmem_alloc(&S.tslot, 512);
+  if (warp == PT_WARPS) tmem_alloc(&S.tslot, 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
 }
 
-// The block's last act: the copies still in flight into its shared memory land and its MMAs
-// complete before it frees the tensor memory (if either does not, it keeps it and only reports).
-// Called after a block barrier that follows the last unit's epilogue: every waiter on `done` is
-// past its phase when the MMA thread commits `done` once more here.
-__device__ __forceinline__ void pol_block_finish(PolSmem& S, uint32_t tbase, int tid, int warp, int lane,
-                                                 PolPhase& ph) {
-  if (tid == 0) {
-    if (ph.last0 >= 0 && !drain_bar(&S.full[0], (ph.last0 >> 1) & 1)) S.no_dealloc = 1;
-    if (ph.last1 >= 0 && !drain_bar(&S.full[1], (ph.last1 >> 1) & 1)) S.no_dealloc = 1;
-  }
-  if (warp == 8 && lane == 0) {
-    mma_commit(&S.done);
-    if (!drain_bar(&S.done, ph.units & 1)) S.no_dealloc = 1;  // every MMA issued here has completed
+// The block's last act: the copies it issued land and its MMAs complete before it frees the tensor memory
+// (if either does not, it keeps it and only reports). The MMAs are waited for on a barrier of their own:
+// after a wait that ran out, `done` may lag any number of phases behind.
+__device__ __forceinline__ void pol_block_finish(PolSmem& S, uint32_t tbase, int warp, PolPhase& ph) {
+  for (int s = 0; s < P_MAXST; ++s)  // (copy thread; the other threads have filled no stage)
+    if ((ph.used >> s & 1) && !drain_bar(&S.fully[s], (ph.uph >> s) & 1)) S.no_dealloc = 1;
+  if (warp == PT_WARPS) {
+    if (elect_one()) mma_commit(&S.fin);
+    __syncwarp();
+    if (!drain_bar(&S.fin, 0)) S.no_dealloc = 1;
+    __syncwarp();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8 && !S.no_dealloc) tmem_dealloc(tbase, 512);
+  if (warp == PT_WARPS && !S.no_dealloc) tmem_dealloc(tbase, 512);
 }
 
-// One work unit per block: the units of one (context, q).
+// The units of one (context, q), dealt to the blocks in turn: one block per SM, so that the copies of the
+// next unit run while the partials of the last one are moved out.
 __global__ void __launch_bounds__(PT_THREADS, 1)
-    k_pol_tc(const __half* __restrict__ YS, const float* __restrict__ wt, int nk, int ni, int ntau, int cpk,
-             int npw, int nstrips, const int4* __restrict__ strips, int nseg, int seg0, int eform,
-             float* __restrict__ part,
-             int* __restrict__ err, long long wait_cycles, int stall) {
+    k_pol_tc(const __grid_constant__ PolJob J, int* __restrict__ err, long long wait_cycles, int stall) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-  PolSmem& S = *reinterpret_cast<PolSmem*>(base + 2 * P_STAGE_BYTES);
+  PolSmem& S = *reinterpret_cast<PolSmem*>(base + P_SMEM);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pol_block_init(S, tid, warp);
   const uint32_t tbase = S.tslot;
-  PolJob J{YS, wt, part, strips, nk, ni, ntau, cpk, npw, nstrips, nseg, seg0, eform, 0};
   PolPhase ph;
-  pol_unit(J, blockIdx.x, S, base, tbase, tid, warp, lane, ph, err, wait_cycles, stall);
-  // the epilogue has seen the unit's `done` phase before the MMA thread commits `done` again in
-  // the finish (two commits completing back to back would move the barrier two phases on)
-  __syncthreads();
-  pol_block_finish(S, tbase, tid, warp, lane, ph);
+  for (int u = blockIdx.x; u < J.units; u += gridDim.x)
+    pol_unit(J, u, S, base, tbase, warp, lane, ph, err, wait_cycles, stall);
+  pol_block_finish(S, tbase, warp, ph);
 }
 
 // The batched form: up to kPolQueueJobs (context, q) jobs, their units numbered one after another;
@@ -387,7 +501,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
                    long long wait_cycles, int stall) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-  PolSmem& S = *reinterpret_cast<PolSmem*>(base + 2 * P_STAGE_BYTES);
+  PolSmem& S = *reinterpret_cast<PolSmem*>(base + P_SMEM);
   __shared__ int item;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pol_block_init(S, tid, warp);
@@ -401,11 +515,12 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
     if (w >= Q.total) break;
     int j = 0, u = w;
     while (j + 1 < Q.njobs && u >= Q.job[j].units) u -= Q.job[j++].units;
-    pol_unit(Q.job[j], u, S, base, tbase, tid, warp, lane, ph, err, wait_cycles, stall);
+    ph.s = 0;  // all stages are free here; the unit's form sets their number and size
+    pol_unit(Q.job[j], u, S, base, tbase, warp, lane, ph, err, wait_cycles, stall);
     __syncthreads();            // every role is done with the unit: the abort flag no longer changes
     if (S.abort_flag) break;    // the same decision in every thread
   }
-  pol_block_finish(S, tbase, tid, warp, lane, ph);
+  pol_block_finish(S, tbase, warp, ph);
 }
 
 // h + l += x with the rounding error of h + x kept exactly in l (Knuth's two-sum)
@@ -720,6 +835,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
       if (last0 >= 0 && !drain_bar(&S.full[0], (last0 >> 1) & 1)) S.no_dealloc = 1;
       if (last1 >= 0 && !drain_bar(&S.full[1], (last1 >> 1) & 1)) S.no_dealloc = 1;
     }
+    __syncwarp();  // the warp meets the block barrier converged
   } else if (warp == MW) {
     // ------------------------------------------------------------ MMA issuer: the warp stays converged
     const uint32_t lead = elect_one();
@@ -735,20 +851,23 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
       const uint32_t arh = st + o, arl = arh + (S_ATILE >> 4), aih = arl + (S_ATILE >> 4), ail = aih + (S_ATILE >> 4);
       const uint32_t urh = st + ((uint32_t)(a_bytes + c0 * 64) >> 4) + o, url = urh + (BT >> 4), vih = url + (BT >> 4),
                      vil = vih + (BT >> 4);
-      // Y1 = Ar U + Ai V
-      mma_f16_warp(y1, arh, urh, dh, id, acc, lead);
-      mma_f16_warp(y1, arh, url, dh, id, 1, lead);
-      mma_f16_warp(y1, arl, urh, dh, id, 1, lead);
-      mma_f16_warp(y1, aih, vih, dh, id, 1, lead);
-      mma_f16_warp(y1, aih, vil, dh, id, 1, lead);
-      mma_f16_warp(y1, ail, vih, dh, id, 1, lead);
-      // Y2 = Ai U - Ar V
-      mma_f16_warp(y2, aih, urh, dh, id, acc, lead);
-      mma_f16_warp(y2, aih, url, dh, id, 1, lead);
-      mma_f16_warp(y2, ail, urh, dh, id, 1, lead);
-      mma_f16_warp(y2, arh, vih, dh, idn, 1, lead);
-      mma_f16_warp(y2, arh, vil, dh, idn, 1, lead);
-      mma_f16_warp(y2, arl, vih, dh, idn, 1, lead);
+      if (lead) {
+        // Y1 = Ar U + Ai V
+        mma_f16_lo(y1, arh, urh, dh, id, acc);
+        mma_f16_lo(y1, arh, url, dh, id, 1);
+        mma_f16_lo(y1, arl, urh, dh, id, 1);
+        mma_f16_lo(y1, aih, vih, dh, id, 1);
+        mma_f16_lo(y1, aih, vil, dh, id, 1);
+        mma_f16_lo(y1, ail, vih, dh, id, 1);
+        // Y2 = Ai U - Ar V
+        mma_f16_lo(y2, aih, urh, dh, id, acc);
+        mma_f16_lo(y2, aih, url, dh, id, 1);
+        mma_f16_lo(y2, ail, urh, dh, id, 1);
+        mma_f16_lo(y2, arh, vih, dh, idn, 1);
+        mma_f16_lo(y2, arh, vil, dh, idn, 1);
+        mma_f16_lo(y2, arl, vih, dh, idn, 1);
+      }
+      __syncwarp();
     };
     for (int u = 0; u < nunit && live; ++u) {
       const int h = u % nh;
@@ -779,14 +898,18 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
             if (c0 < NC) step(st, 2 * ks, c0, NC - c0, 1);
           }
         }
-        mma_commit_warp(&S.empty[s], lead);
-        mma_commit_warp(&S.col[kc], lead);
+        if (lead) {
+          mma_commit(&S.empty[s]);
+          mma_commit(&S.col[kc]);
+        }
+        __syncwarp();
         s ^= 1;
         ph ^= s ^ 1;  // the phase turns when stage 0 comes round
         if (!live) break;
       }
     }
-    mma_commit_warp(&S.fin, lead);
+    if (lead) mma_commit(&S.fin);
+    __syncwarp();
     if (!drain_bar(&S.fin, 0)) S.no_dealloc = 1;  // every MMA issued here has completed
     __syncwarp();
   } else {
@@ -904,6 +1027,7 @@ struct PolPrep {
   int nstrips = 0, nseg = 0, seg_pass = 0, base_units = 0, nb32 = 0, cpk = 0, npw = 0, eform = 1;
   float* d_part = nullptr;
   float* d_wt = nullptr;
+  float* d_xf = nullptr;
   __half* d_ys = nullptr;
   double* d_e = nullptr;
   int4* d_strips = nullptr;
@@ -945,20 +1069,22 @@ static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
   while (base_units * nseg < 2 * sms && (total + nseg) / (nseg + 1) >= 4) ++nseg;
   // the partials of at most pol_part_bytes are held at once: segments run in passes, each
   // reduced into P (the first pass writes, later ones add)
-  const size_t seg_bytes = (size_t)base_units * (eform ? 1 : 2) * P_TILE * sizeof(float);
+  const size_t seg_bytes = (size_t)base_units * (eform ? 1 : 2) * P_TILE * sizeof(float);  // E form: units of two tau
   const int seg_pass = (int)std::max<size_t>(1, std::min<size_t>(nseg, c->pol_part_bytes / seg_bytes));
   const size_t part_bytes = seg_bytes * seg_pass;
   const size_t wt_bytes = (size_t)c->nk * c->ntau * npw * sizeof(float);
   const size_t ys_bytes = (size_t)c->nk * cpk * nib * 2 * 128 * 64 * sizeof(__half);
+  const size_t xf_bytes = eform ? (size_t)c->nk * cpk * nib * 2 * 128 * 32 * sizeof(float) : 0;
   const size_t e_bytes = eform ? (size_t)c->ntau * ni * ni * sizeof(double) : 0;
   gw_status st;
-  if ((st = ensure(c, &c->mw.wslices, &c->mw.wslices_bytes, part_bytes + wt_bytes + ys_bytes + e_bytes,
+  if ((st = ensure(c, &c->mw.wslices, &c->mw.wslices_bytes, part_bytes + wt_bytes + ys_bytes + xf_bytes + e_bytes,
                    "P workspace")) != GW_OK)
     return st;
   float* d_part = (float*)c->mw.wslices;
   float* d_wt = d_part + part_bytes / sizeof(float);
   __half* d_ys = (__half*)((char*)d_wt + wt_bytes);
-  double* d_e = (double*)((char*)d_ys + ys_bytes);
+  float* d_xf = (float*)((char*)d_ys + ys_bytes);
+  double* d_e = (double*)((char*)d_xf + xf_bytes);
   const size_t meta_bytes = sizeof(int4) * strips.size() + sizeof(int) * strip_of.size();
   const void* meta_before = c->mw.dacc;
   if ((st = ensure(c, (void**)&c->mw.dacc, &c->mw.dacc_bytes, meta_bytes + 256, "P strips")) != GW_OK) return st;
@@ -973,11 +1099,11 @@ static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
     c->mw.strips_ready = true;
     c->mw.strips_form = eform;
   }
-  if (ni % 128) cudaMemsetAsync(d_ys, 0, ys_bytes, c->stream);  // rows >= ni of the last block stay zero
+  // rows >= ni of the last block stay as they are: they reach only rows of the strips that nothing reads
   const double2* Mq = (const double2*)m_block(c, iq);
   if (!Mq) return GW_ECUDA;
   const int64_t nsp = (int64_t)c->nk * ni * cpk * 4;
-  k_split_y<<<(unsigned)((nsp + 255) / 256), 256, 0, c->stream>>>(Mq, c->nk, ni, np, cpk, nib, d_ys);
+  k_split_y<<<(unsigned)((nsp + 255) / 256), 256, 0, c->stream>>>(Mq, c->nk, ni, np, cpk, nib, eform, d_ys, d_xf);
   if ((st = check_launch(c, "split_y")) != GW_OK) return st;
   const int64_t nwt = (int64_t)c->nk * c->ntau * npw;
   k_pol_weights<<<(unsigned)((nwt + 255) / 256), 256, 0, c->stream>>>(G, c->d_kmq + (size_t)iq * c->nk, c->nk, c->nb,
@@ -993,6 +1119,7 @@ static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
   pp->d_part = d_part;
   pp->d_wt = d_wt;
   pp->d_ys = d_ys;
+  pp->d_xf = d_xf;
   pp->d_e = d_e;
   pp->d_strips = d_strips;
   pp->d_strip_of = d_strip_of;
@@ -1019,7 +1146,12 @@ static gw_status pol_reduce(gw_ctx* c, const PolPrep& pp, int s0, int ns, double
   return check_launch(c, "pol_form");
 }
 
-static size_t pol_smem() { return 1024 + 2 * P_STAGE_BYTES + sizeof(PolSmem); }
+static size_t pol_smem() { return 1024 + P_SMEM + sizeof(PolSmem); }
+
+static PolJob pol_job(const gw_ctx* c, const PolPrep& pp, int s0, int ns) {
+  return PolJob{pp.d_ys, pp.d_xf, pp.d_wt, pp.d_part, pp.d_strips, c->nk, c->ni, c->ntau, pp.cpk, pp.npw,
+                pp.nstrips, pp.nseg, s0, pp.eform, pp.base_units / (pp.eform ? 2 : 1) * ns};
+}
 
 gw_status launch_pol_mixed(gw_ctx* c, int iq, const double* G, int prec, double* P) {
   if (prec != GW_FP16X2) return set_err(c, GW_EUNSUPPORTED, "polarization: only GW_FP16X2 is built on tensor cores");
@@ -1031,10 +1163,8 @@ gw_status launch_pol_mixed(gw_ctx* c, int iq, const double* G, int prec, double*
   for (int s0 = 0; s0 < pp.nseg; s0 += pp.seg_pass) {
     const int ns = std::min(pp.seg_pass, pp.nseg - s0);
     kt_begin(c, "k_pol_tc");
-    k_pol_tc<<<pp.base_units * ns, PT_THREADS, smem, c->stream>>>(pp.d_ys, pp.d_wt, c->nk, c->ni, c->ntau, pp.cpk,
-                                                                  pp.npw, pp.nstrips, pp.d_strips, pp.nseg, s0,
-                                                                  pp.eform, pp.d_part, c->d_err, c->wait_cycles,
-                                                                  c->fault_stall);
+    const PolJob J = pol_job(c, pp, s0, ns);
+    k_pol_tc<<<std::min(J.units, num_sms(c)), PT_THREADS, smem, c->stream>>>(J, c->d_err, c->wait_cycles, c->fault_stall);
     kt_end(c);
     if ((st = check_launch(c, "pol_tc")) != GW_OK) return st;
     if ((st = pol_reduce(c, pp, s0, ns, P)) != GW_OK) return st;
@@ -1069,8 +1199,7 @@ gw_status launch_pol_many(int njobs, gw_ctx* const* ctxs, const int* iqs, const 
       const int ns = std::min(pp[j].seg_pass, pp[j].nseg - s0[j]);
       gw_ctx* c = ctxs[j];
       PolJob& J = Q.job[Q.njobs++];
-      J = PolJob{pp[j].d_ys, pp[j].d_wt, pp[j].d_part, pp[j].d_strips, c->nk, c->ni, c->ntau, pp[j].cpk,
-                 pp[j].npw, pp[j].nstrips, pp[j].nseg, s0[j], pp[j].eform, pp[j].base_units * ns};
+      J = pol_job(c, pp[j], s0[j], ns);
       Q.total += J.units;
       jid.push_back(j);
       nsj.push_back(ns);

@@ -132,3 +132,33 @@ def test_captured_without_workspace(gw):
     assert float((P - P1).abs().max()) <= 128 * 2.0 ** -52 * float(P1.abs().max())
     assert float((S - S1).abs().max()) <= 128 * 2.0 ** -52 * float(S1.abs().max())
     ctx.close()
+
+
+def test_stalled_pipeline_reports_and_recovers(gw):
+    """The digit GEMM's waits are bounded like the mixed kernels': an injected stall (1 ms budget) is reported by
+    gw_sync, and the same context then gives the healthy values again, bit for bit."""
+    torch, rng, cr, gr, M, ctx, G, occ = _setup(gw, 2, 6, 96, 8, 12)
+    X = rng.standard_normal((8, 96, 96))
+    W = torch.from_numpy(np.ascontiguousarray(X + np.swapaxes(X, 1, 2)) + 0j).cuda()
+    Gd = torch.from_numpy(G).cuda()
+
+    def run():
+        P = torch.zeros(8, 96, 96, dtype=torch.complex128, device="cuda")
+        S = torch.zeros(2, 6, 8, dtype=torch.float64, device="cuda")
+        ctx.polarization(0, Gd, P, gw.GW_FP64)
+        ctx.selfenergy(0, Gd, None, W, S, None, gw.GW_FP64)
+        return P, S
+
+    P0, S0 = run()
+    ctx.sync()
+    ctx.set_tuning(gw.GW_TUNE_WAIT_CYCLES, 2_000_000)
+    ctx.set_tuning(gw.GW_TUNE_FAULT_STALL, 1)
+    run()
+    with pytest.raises(gw.GwError, match="GW_ETIMEOUT"):
+        ctx.sync()
+    ctx.set_tuning(gw.GW_TUNE_FAULT_STALL, 0)
+    ctx.set_tuning(gw.GW_TUNE_WAIT_CYCLES, 4_000_000_000)
+    P1, S1 = run()
+    ctx.sync()
+    assert torch.equal(P0, P1) and torch.equal(S0, S1)
+    ctx.close()
