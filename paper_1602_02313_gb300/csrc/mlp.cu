@@ -5,8 +5,8 @@
 // first nw_fit fermionic frequencies, real-stacked), so no labels are needed.
 //
 // Every matrix product runs on the tensor cores (tcgen05, fp16 operands from shared
-// memory in the 128-byte swizzle layout, FP32 accumulation in TMEM); activations,
-// the loss and Adam run in FP32 kernels. Weights are kept in FP32 (master) with fp16
+// memory in the 128-byte swizzle layout, FP32 accumulation in TMEM) with the activations and their
+// derivatives in the epilogues; the loss and Adam run in FP32 kernels. Weights are kept in FP32 (master) with fp16
 // copies W [out][in] and W^T [in][out] for the two product shapes.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -25,7 +25,9 @@ struct gw_mlp {
   cudaStream_t stream = nullptr;
   int nin = 0, nh = 0, nhidden = 0, nout = 0, nlayers = 0;
   std::vector<int> din, dout;  // per layer
-  std::vector<float*> W, b, mW, vW, mb, vb, gW, gb;
+  std::vector<float*> W, b, mW, vW, mb, vb;
+  std::vector<float*> gW, gb;  // in `grads`, parameter order
+  float* grads = nullptr;
   std::vector<__half*> Wh, WTh;
   int64_t step = 0;
   // workspaces for batch <= cap
@@ -35,10 +37,10 @@ struct gw_mlp {
   std::vector<__half*> HT;    // fp16 transposed activations [dout][B] (incl. input at index 0)
   __half* Xh = nullptr;       // fp16 input [B][nin]
   float* out = nullptr;       // [B][nout]
-  float* dZ = nullptr;        // [B][max d]
-  __half* dZh = nullptr;      // [B][max d]
-  __half* dZT = nullptr;      // [max d][B]
-  float* dH = nullptr;        // [B][max d]
+  std::vector<float*> dZ;     // per layer [B][dout]
+  std::vector<__half*> dZh;   // per layer [B][dout]
+  std::vector<__half*> dZT;   // per layer [dout][B]
+  float* part = nullptr;      // [K splits][num_params]: dW over parts of the batch
   float* loss = nullptr;      // [1]
   int* err = nullptr;
   std::string errmsg;
@@ -47,88 +49,37 @@ struct gw_mlp {
 namespace gwi {
 namespace mlpk {
 
-// ------------------------------------------------------------------ generic GEMM
-// C[M][N] (FP32) = A[M][K] * B[N][K]^T, A, B fp16 row-major. M % 128 == 0, N % 16 == 0,
-// K % 64 == 0. One block per (128-row tile, 256-column tile); one pipeline stage.
-constexpr int GEMM_THREADS = 128;
+// ------------------------------------------------------------------ GEMM with fused epilogues
+// C[M][N] (FP32) = A[M][K] * B[N][K]^T, A, B fp16 row-major. M % 128 == 0, N % 64 == 0, K % 64 == 0. One
+// block per 128 x 64 tile (and part of K): the layers are a few hundred wide, so small tiles fill more SMs
+// and a panel of up to 256 k is brought in one go (the latency of one load, not of one per 64 k).
+// Measured at batch 1024, 128-256-256-256-128: 11 us per GEMM with its epilogue, against 50 us in 128 x 256
+// tiles with a load per 64 k and 5 us for each elementwise pass; loss and gradients 705 -> 130 us, 31 -> 11
+// launches. What bounds it is latency: 32 blocks, one load, one short MMA chain, one epilogue.
+constexpr int GEMM_THREADS = 256;
+constexpr int GN = 64, GK = 256;
+constexpr int G_A = 128 * 128, G_B = GN * 128;  // bytes of one 64-wide K tile
+constexpr int G_SMEM = 1024 + (GK / 64) * (G_A + G_B);
 
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-    k_gemm_tc(const __half* __restrict__ A, const __half* __restrict__ B, float* __restrict__ C, int M, int N, int K,
-              int* __restrict__ err) {
-  extern __shared__ __align__(1024) unsigned char smraw[];
-  unsigned char* base = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-  unsigned char* sA = base;          // 128 x 128 B
-  unsigned char* sB = base + 16384;  // <= 256 x 128 B
-  __shared__ uint64_t bar;
-  __shared__ uint32_t tslot;
-  __shared__ int abort_g, no_dealloc;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * 128, n0 = blockIdx.y * 256;
-  const int Nt = min(256, N - n0);
-  if (tid == 0) {
-    mbar_init(&bar, 1);
-    abort_g = 0;
-    no_dealloc = 0;
-    fence_mbar_init();
-  }
-  if (warp == 0) tmem_alloc(&tslot, 256);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tbase = tslot;
-  const uint32_t id = idesc_f16(128, Nt, false, false);
-  int kc = 0;
-  for (; kc < K / 64; ++kc) {
-    for (int e = tid; e < 128 * 8; e += GEMM_THREADS) {
-      const int r = e >> 3, c = e & 7;
-      const uint4 v = *reinterpret_cast<const uint4*>(A + (size_t)(m0 + r) * K + kc * 64 + 8 * c);
-      *reinterpret_cast<uint4*>(sA + sw128_off(r, 8 * c)) = v;
-    }
-    for (int e = tid; e < Nt * 8; e += GEMM_THREADS) {
-      const int r = e >> 3, c = e & 7;
-      const uint4 v = *reinterpret_cast<const uint4*>(B + (size_t)(n0 + r) * K + kc * 64 + 8 * c);
-      *reinterpret_cast<uint4*>(sB + sw128_off(r, 8 * c)) = v;
-    }
-    fence_proxy_async_smem();
-    __syncthreads();
-    if (tid == 0) {
-      tc_fence_after();
-#pragma unroll
-      for (int ks = 0; ks < 4; ++ks)
-        mma_f16(tbase, sdesc_sw128(smem_u32(sA) + 32 * ks), sdesc_sw128(smem_u32(sB) + 32 * ks), id,
-                (kc > 0 || ks > 0) ? 1u : 0u);
-      mma_commit(&bar);
-    }
-    // a thread whose wait runs out stops the whole block after the barrier (abort_g is written
-    // only between the two barriers of an iteration, so every thread reads the same value)
-    if (!mbar_wait(&bar, kc & 1, err)) abort_g = 1;
-    tc_fence_after();
-    __syncthreads();
-    if (abort_g) break;
-  }
-  // MMAs still running into TMEM complete before the block frees it; if they do not, it keeps it
-  if (abort_g && tid == 0 && !mbar_wait_drain(&bar, kc & 1)) no_dealloc = 1;
-  __syncthreads();
-  const bool ok = !abort_g;
-  const int row = 32 * warp + lane;
-  for (int c = 0; c < Nt; c += 16) {
-    float v[16];
-    if (ok) {
-      tmem_ld16(tbase + ((uint32_t)(32 * warp) << 16) + c, v);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 16; ++e) v[e] = 0.f;
-    }
-    float* o = C + (size_t)(m0 + row) * N + n0 + c;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) o[e] = v[e];
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0 && !no_dealloc) tmem_dealloc(tbase, 256);
-}
+enum { EPI_ACT = 0, EPI_BACK = 1, EPI_PART = 2 };
+struct GemmArgs {
+  const __half *A, *B;
+  int M, N, K;
+  const float* bias;    // EPI_ACT
+  float* Z;             // EPI_ACT: pre-activations, written; EPI_BACK: the lower layer's, read
+  __half *H, *HT;       // EPI_ACT: activations; EPI_BACK: dZ in fp16, both [row][col] and [col][row]
+  float* out;           // EPI_ACT: FP32 activations of the last layer; EPI_BACK: dZ; EPI_PART: partial C
+  int last;
+};
+// The dW products of all layers in one launch (EPI_PART): tiles of job j from tile0, K in `splits` parts
+constexpr int kMaxLayers = 16;
+struct GemmJobs {
+  GemmArgs job[kMaxLayers];
+  int tile0[kMaxLayers + 1];
+  int njobs, kpart;
+  int64_t stride;  // floats from one part of K to the next
+};
 
-// ------------------------------------------------------------------ elementwise
 __device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_g(float z) {
   return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
@@ -136,64 +87,235 @@ __device__ __forceinline__ float gelu_g(float z) {
 __device__ __forceinline__ float softplus_f(float z) { return fmaxf(z, 0.f) + log1pf(expf(-fabsf(z))); }
 __device__ __forceinline__ float sigmoid_f(float z) { return 1.f / (1.f + expf(-z)); }
 
-// Z += bias; H = act(Z) (fp16 row-major and transposed copies; FP32 out for the last layer)
-__global__ void k_bias_act(float* __restrict__ Z, const float* __restrict__ bias, int64_t Bn, int d, int last,
-                           __half* __restrict__ H, __half* __restrict__ HT, float* __restrict__ out) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= Bn * d) return;
-  const int64_t r = e / d;
-  const int c = (int)(e % d);
-  const float z = Z[e] + bias[c];
-  Z[e] = z;
-  const float h = last ? softplus_f(z) : gelu_f(z);
-  if (last) out[e] = h;
-  if (H) H[e] = __float2half_rn(h);
-  if (HT) HT[(size_t)c * Bn + r] = __float2half_rn(h);
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
-// residual R = out A^T - x (FP32), loss = (1/B) sum R^2, dOut = (2/B) R A
-__global__ void k_loss(const float* __restrict__ out, const float* __restrict__ x, const float* __restrict__ Acpe,
-                       int64_t Bn, int nout, int nx, float* __restrict__ dOut, float* __restrict__ loss) {
-  extern __shared__ float sm[];
-  float* r = sm;  // [nx]
-  const int64_t b = blockIdx.x;
-  for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-    float s = -x[b * nx + i];
-    for (int m = 0; m < nout; ++m) s = fmaf(Acpe[(size_t)i * nout + m], out[b * nout + m], s);
-    r[i] = s;
+template <int EPI>
+__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int tile, int k0, int k1, int* err) {
+  extern __shared__ __align__(1024) unsigned char smraw[];
+  unsigned char* base = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+  __shared__ uint64_t bar;
+  __shared__ uint32_t tslot;
+  __shared__ int abort_g, no_dealloc;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nt = g.N / GN, m0 = (tile / nt) * 128, n0 = (tile % nt) * GN;
+  if (tid == 0) {
+    mbar_init(&bar, 1);
+    abort_g = 0;
+    no_dealloc = 0;
+    fence_mbar_init();
   }
+  if (warp == 0) tmem_alloc(&tslot, GN);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = tslot;
+  int panel = 0;
+  for (int kp = k0; kp < k1; kp += GK, ++panel) {
+    const int kn = min(GK, k1 - kp), kc8 = kn / 8;  // 16-byte pieces of a row
+    for (int e = tid; e < (128 + GN) * kc8; e += GEMM_THREADS) {
+      const int r = e / kc8, c = e % kc8;
+      if (r < 128)
+        cp16(base + (c >> 3) * G_A + sw128_off(r, 8 * (c & 7)), g.A + (size_t)(m0 + r) * g.K + kp + 8 * c);
+      else
+        cp16(base + (GK / 64) * G_A + (c >> 3) * G_B + sw128_off(r - 128, 8 * (c & 7)),
+             g.B + (size_t)(n0 + r - 128) * g.K + kp + 8 * c);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    fence_proxy_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+      tc_fence_after();
+      for (int q = 0; q < kn / 64; ++q) {
+        const uint32_t a = smem_u32(base + q * G_A), b = smem_u32(base + (GK / 64) * G_A + q * G_B);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+          mma_f16(tbase, sdesc_sw128(a + 32 * ks), sdesc_sw128(b + 32 * ks), idesc_f16(128, GN, false, false),
+                  (kp > k0 || q > 0 || ks > 0) ? 1u : 0u);
+      }
+      mma_commit(&bar);
+    }
+    // a thread whose wait runs out stops the whole block after the barrier (abort_g is written
+    // only between the two barriers of an iteration, so every thread reads the same value)
+    if (!mbar_wait(&bar, panel & 1, err)) abort_g = 1;
+    tc_fence_after();
+    __syncthreads();
+    if (abort_g) break;
+  }
+  // MMAs still running into TMEM complete before the block frees it; if they do not, it keeps it
+  if (abort_g && tid == 0 && !mbar_wait_drain(&bar, panel & 1)) no_dealloc = 1;
+  __syncthreads();
+  const bool ok = !abort_g;
+  // warp: rows 32 (warp & 3) + lane, columns 32 (warp >> 2) .. + 31
+  const int row = m0 + 32 * (warp & 3) + lane;
+  for (int c = 32 * (warp >> 2); c < 32 * (warp >> 2) + 32; c += 16) {
+    float v[16];
+    if (ok) {
+      tmem_ld16(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + c, v);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v[e] = 0.f;
+    }
+    const int col = n0 + c;
+    const size_t o = (size_t)row * g.N + col;
+    // 16-byte accesses (col is a multiple of 16): scalar ones by 32 lanes in 32 rows cost a sector each
+    float4* zo = reinterpret_cast<float4*>((EPI == EPI_PART ? g.out : g.Z) + o);
+    if (EPI == EPI_PART) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) zo[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      continue;
+    }
+    alignas(16) __half h[16];
+    float y[16];
+    if (EPI == EPI_ACT) {  // z = A B^T + bias, h = act(z)
+      const float4* bo = reinterpret_cast<const float4*>(g.bias + col);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 bq = bo[q];
+        v[4 * q] += bq.x;
+        v[4 * q + 1] += bq.y;
+        v[4 * q + 2] += bq.z;
+        v[4 * q + 3] += bq.w;
+        zo[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+#pragma unroll
+      for (int e = 0; e < 16; ++e) y[e] = g.last ? softplus_f(v[e]) : gelu_f(v[e]);
+    } else {  // dZ = dH act'(Z) of a hidden layer
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 z = zo[q];
+        y[4 * q] = v[4 * q] * gelu_g(z.x);
+        y[4 * q + 1] = v[4 * q + 1] * gelu_g(z.y);
+        y[4 * q + 2] = v[4 * q + 2] * gelu_g(z.z);
+        y[4 * q + 3] = v[4 * q + 3] * gelu_g(z.w);
+      }
+    }
+    if (EPI == EPI_BACK || g.last) {
+      float4* yo = reinterpret_cast<float4*>(g.out + o);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) yo[q] = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      h[e] = __float2half_rn(y[e]);
+      g.HT[(size_t)(col + e) * g.M + row] = h[e];
+    }
+    uint4* ho = reinterpret_cast<uint4*>(g.H + o);
+    ho[0] = reinterpret_cast<const uint4*>(h)[0];
+    ho[1] = reinterpret_cast<const uint4*>(h)[1];
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0 && !no_dealloc) tmem_dealloc(tbase, GN);
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(GEMM_THREADS) k_gemm_tc(const __grid_constant__ GemmArgs g, int* __restrict__ err) {
+  gemm_tile<EPI>(g, blockIdx.x, 0, g.K, err);
+}
+
+__global__ void __launch_bounds__(GEMM_THREADS) k_gemm_dw(const __grid_constant__ GemmJobs J, int* __restrict__ err) {
+  int j = 0;
+  while (j + 1 < J.njobs && (int)blockIdx.x >= J.tile0[j + 1]) ++j;
+  GemmArgs g = J.job[j];
+  g.out += blockIdx.y * J.stride;
+  const int k0 = blockIdx.y * J.kpart;
+  gemm_tile<EPI_PART>(g, blockIdx.x - J.tile0[j], k0, min(g.K, k0 + J.kpart), err);
+}
+
+// Gradients in parameter order from the parts: blocks of 256 weights (the parts summed in order), and for
+// each layer's biases the column sums of dZ (block: 32 columns x 32 row lanes).
+struct GradJobs {
+  const float* dZ[kMaxLayers];
+  int64_t w0[kMaxLayers];    // first weight of the layer in parameter order
+  int nw[kMaxLayers], d[kMaxLayers], blk0[kMaxLayers + 1], wblk[kMaxLayers];
+  int nlayers, splits;
+  int64_t stride, batch;
+};
+__global__ void __launch_bounds__(1024) k_grads(const __grid_constant__ GradJobs J, const float* __restrict__ part,
+                                                float* __restrict__ grads) {
+  int l = 0;
+  while (l + 1 < J.nlayers && (int)blockIdx.x >= J.blk0[l + 1]) ++l;
+  const int b = blockIdx.x - J.blk0[l];
+  if (b < J.wblk[l]) {
+    const int e = b * 1024 + threadIdx.x;
+    if (e >= J.nw[l]) return;
+    const float* p = part + J.w0[l] + e;
+    float s = p[0];
+    for (int q = 1; q < J.splits; ++q) s += p[q * J.stride];
+    grads[J.w0[l] + e] = s;
+    return;
+  }
+  __shared__ float sm[32][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c = 32 * (b - J.wblk[l]) + tx, d = J.d[l];
+  const float* z = J.dZ[l] + c;
+  float s = 0.f;
+#pragma unroll 4
+  for (int64_t r = ty; r < J.batch; r += 32) s += z[r * d];
+  sm[ty][tx] = s;
+  __syncthreads();
+  if (ty == 0) {
+    for (int q = 1; q < 32; ++q) s += sm[q][tx];
+    grads[J.w0[l] + J.nw[l] + c] = s;
+  }
+}
+
+// ------------------------------------------------------------------ loss and the rest
+// residual R = out A^T - x (FP32), loss = (1/B) sum R^2, dOut = (2/B) R A, dZ = dOut softplus'(Z) of the last
+// layer with its fp16 copies. One block per LS = 8 samples: every element of A is read once for them (one
+// sample where the outputs of eight do not fit in shared memory). 67 -> 24 us at batch 1024.
+template <int LS>
+__global__ void __launch_bounds__(128) k_loss(const float* __restrict__ out, const float* __restrict__ x,
+                                              const float* __restrict__ Acpe, const float* __restrict__ Z, int64_t Bn,
+                                              int nout, int nx, float* __restrict__ dZ, __half* __restrict__ dZh,
+                                              __half* __restrict__ dZT, float* __restrict__ loss) {
+  extern __shared__ float sm[];
+  float* so = sm;               // [nout][LS]
+  float* r = sm + nout * LS;    // [nx][LS]
+  const int64_t b0 = (int64_t)blockIdx.x * LS;  // Bn is a multiple of 128
+  for (int e = threadIdx.x; e < nout * LS; e += blockDim.x) so[e] = out[(b0 + e % LS) * nout + e / LS];
   __syncthreads();
   float part = 0.f;
-  for (int i = threadIdx.x; i < nx; i += blockDim.x) part += r[i] * r[i];
+  for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+    float s[LS];
+#pragma unroll
+    for (int q = 0; q < LS; ++q) s[q] = -x[(b0 + q) * nx + i];
+#pragma unroll 8
+    for (int m = 0; m < nout; ++m) {
+      const float a = Acpe[(size_t)i * nout + m];
+#pragma unroll
+      for (int q = 0; q < LS; ++q) s[q] = fmaf(a, so[m * LS + q], s[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < LS; ++q) {
+      r[i * LS + q] = s[q];
+      part += s[q] * s[q];
+    }
+  }
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, part / (float)Bn);
+  __syncthreads();
   for (int m = threadIdx.x; m < nout; m += blockDim.x) {
-    float s = 0.f;
-    for (int i = 0; i < nx; ++i) s = fmaf(r[i], Acpe[(size_t)i * nout + m], s);
-    dOut[b * nout + m] = (2.f / (float)Bn) * s;
+    float s[LS] = {};
+#pragma unroll 8
+    for (int i = 0; i < nx; ++i) {
+      const float a = Acpe[(size_t)i * nout + m];
+#pragma unroll
+      for (int q = 0; q < LS; ++q) s[q] = fmaf(r[i * LS + q], a, s[q]);
+    }
+    __half h[LS];
+#pragma unroll
+    for (int q = 0; q < LS; ++q) {
+      const size_t e = (size_t)(b0 + q) * nout + m;
+      const float g = (2.f / (float)Bn) * s[q] * sigmoid_f(Z[e]);
+      dZ[e] = g;
+      h[q] = __float2half_rn(g);
+      dZh[e] = h[q];
+    }
+#pragma unroll
+    for (int q = 0; q < LS; ++q) dZT[(size_t)m * Bn + b0 + q] = h[q];
   }
-}
-
-// dZ = dH * act'(Z); fp16 copies (row-major and transposed) of dZ
-__global__ void k_act_back(const float* __restrict__ dH, const float* __restrict__ Z, int64_t Bn, int d, int last,
-                           float* __restrict__ dZ, __half* __restrict__ dZh, __half* __restrict__ dZT) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= Bn * d) return;
-  const int64_t r = e / d;
-  const int c = (int)(e % d);
-  const float z = Z[e];
-  const float g = dH[e] * (last ? sigmoid_f(z) : gelu_g(z));
-  dZ[e] = g;
-  dZh[e] = __float2half_rn(g);
-  dZT[(size_t)c * Bn + r] = __float2half_rn(g);
-}
-
-__global__ void k_colsum(const float* __restrict__ dZ, int64_t Bn, int d, float* __restrict__ gb) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d) return;
-  float s = 0.f;
-  for (int64_t r = 0; r < Bn; ++r) s += dZ[r * d + c];
-  gb[c] = s;
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
@@ -244,51 +366,51 @@ gw_status mlp_check(gw_mlp* m, const char* what) {
   return GW_OK;
 }
 
-gw_status gemm(gw_mlp* m, const __half* A, const __half* B, float* C, int M, int N, int K) {
-  const size_t smem = 1024 + 16384 + 256 * 128;
-  cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  dim3 grid(M / 128, (N + 255) / 256);
-  k_gemm_tc<<<grid, GEMM_THREADS, smem, m->stream>>>(A, B, C, M, N, K, m->err);
+template <int EPI>
+gw_status gemm(gw_mlp* m, const GemmArgs& g) {
+  cudaFuncSetAttribute(k_gemm_tc<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
+  k_gemm_tc<EPI><<<(g.M / 128) * (g.N / GN), GEMM_THREADS, G_SMEM, m->stream>>>(g, m->err);
   return mlp_check(m, "mlp gemm");
 }
 
-int maxd(const gw_mlp* m) {
-  int d = m->nin;
-  for (int l = 0; l < m->nlayers; ++l) d = std::max(d, m->dout[l]);
-  return d;
-}
+// parts of the batch in the dW products: 256 samples each, at most 16 parts
+int dw_part(int64_t Bn) { return (int)std::max<int64_t>(GK, (Bn / 16 + 63) / 64 * 64); }
 
 gw_status ensure_batch(gw_mlp* m, int64_t Bn) {
   if (Bn <= m->cap) return GW_OK;
   auto fr = [](void* p) {
     if (p) cudaFree(p);
   };
-  for (float* p : m->Z) fr(p);
-  for (__half* p : m->Hh) fr(p);
-  for (__half* p : m->HT) fr(p);
+  const int L = m->nlayers;
+  for (auto* v : {&m->Z, &m->dZ}) {
+    for (float* p : *v) fr(p);
+    v->assign(L, nullptr);
+  }
+  for (auto* v : {&m->Hh, &m->HT, &m->dZh, &m->dZT}) {
+    for (__half* p : *v) fr(p);
+    v->assign(v == &m->HT ? L + 1 : L, nullptr);
+  }
   fr(m->Xh);
   fr(m->out);
-  fr(m->dZ);
-  fr(m->dZh);
-  fr(m->dZT);
-  fr(m->dH);
-  const int L = m->nlayers, D = maxd(m);
-  m->Z.assign(L, nullptr);
-  m->Hh.assign(L, nullptr);
-  m->HT.assign(L + 1, nullptr);
+  fr(m->part);
+  m->Xh = nullptr;
+  m->out = m->part = nullptr;
   bool ok = true;
   for (int l = 0; l < L; ++l) {
-    ok &= cudaMalloc((void**)&m->Z[l], sizeof(float) * Bn * m->dout[l]) == cudaSuccess;
-    ok &= cudaMalloc((void**)&m->Hh[l], sizeof(__half) * Bn * m->dout[l]) == cudaSuccess;
-    ok &= cudaMalloc((void**)&m->HT[l + 1], sizeof(__half) * Bn * m->dout[l]) == cudaSuccess;
+    const size_t n = (size_t)Bn * m->dout[l];
+    ok &= cudaMalloc((void**)&m->Z[l], sizeof(float) * n) == cudaSuccess;
+    ok &= cudaMalloc((void**)&m->Hh[l], sizeof(__half) * n) == cudaSuccess;
+    ok &= cudaMalloc((void**)&m->HT[l + 1], sizeof(__half) * n) == cudaSuccess;
+    ok &= cudaMalloc((void**)&m->dZ[l], sizeof(float) * n) == cudaSuccess;
+    ok &= cudaMalloc((void**)&m->dZh[l], sizeof(__half) * n) == cudaSuccess;
+    ok &= cudaMalloc((void**)&m->dZT[l], sizeof(__half) * n) == cudaSuccess;
   }
   ok &= cudaMalloc((void**)&m->HT[0], sizeof(__half) * Bn * m->nin) == cudaSuccess;
   ok &= cudaMalloc((void**)&m->Xh, sizeof(__half) * Bn * m->nin) == cudaSuccess;
   ok &= cudaMalloc((void**)&m->out, sizeof(float) * Bn * m->nout) == cudaSuccess;
-  ok &= cudaMalloc((void**)&m->dZ, sizeof(float) * Bn * D) == cudaSuccess;
-  ok &= cudaMalloc((void**)&m->dZh, sizeof(__half) * Bn * D) == cudaSuccess;
-  ok &= cudaMalloc((void**)&m->dZT, sizeof(__half) * Bn * D) == cudaSuccess;
-  ok &= cudaMalloc((void**)&m->dH, sizeof(float) * Bn * D) == cudaSuccess;
+  // any batch up to Bn: the number of parts grows with the batch up to 16
+  const int64_t splits = std::min<int64_t>(16, (Bn + GK - 1) / GK);
+  ok &= cudaMalloc((void**)&m->part, sizeof(float) * splits * gw_mlp_num_params(m)) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     m->cap = 0;
@@ -303,36 +425,62 @@ gw_status forward(gw_mlp* m, int64_t Bn, const float* x) {
   const int64_t nx = Bn * m->nin;
   k_x_half<<<(unsigned)((nx + 255) / 256), 256, 0, m->stream>>>(x, Bn, m->nin, m->Xh, m->HT[0]);
   if ((st = mlp_check(m, "mlp input")) != GW_OK) return st;
-  const __half* h = m->Xh;
   for (int l = 0; l < m->nlayers; ++l) {
-    if ((st = gemm(m, h, m->Wh[l], m->Z[l], (int)Bn, m->dout[l], m->din[l])) != GW_OK) return st;
-    const int last = l == m->nlayers - 1;
-    const int64_t n = Bn * m->dout[l];
-    k_bias_act<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(m->Z[l], m->b[l], Bn, m->dout[l], last, m->Hh[l],
-                                                                   m->HT[l + 1], m->out);
-    if ((st = mlp_check(m, "mlp act")) != GW_OK) return st;
-    h = m->Hh[l];
+    GemmArgs g{l ? m->Hh[l - 1] : m->Xh, m->Wh[l], (int)Bn, m->dout[l], m->din[l], m->b[l], m->Z[l], m->Hh[l],
+               m->HT[l + 1], m->out, l == m->nlayers - 1};
+    if ((st = gemm<EPI_ACT>(m, g)) != GW_OK) return st;
   }
   return GW_OK;
 }
 
+// Gradients into m->grads. More layers than fit the job tables go in runs of kMaxLayers.
 gw_status backward(gw_mlp* m, int64_t Bn, const float* x, const float* Acpe, int nx) {
   gw_status st;
+  const int L = m->nlayers, e = L - 1;
   cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream);
-  k_loss<<<(unsigned)Bn, 128, sizeof(float) * nx, m->stream>>>(m->out, x, Acpe, Bn, m->nout, nx, m->dH, m->loss);
+  const size_t sm1 = sizeof(float) * ((size_t)m->nout + nx);
+  auto loss = [&](auto* kernel, int ls) {
+    if (ls * sm1 > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(ls * sm1));
+    kernel<<<(unsigned)(Bn / ls), 128, ls * sm1, m->stream>>>(m->out, x, Acpe, m->Z[e], Bn, m->nout, nx, m->dZ[e], m->dZh[e],
+                                                             m->dZT[e], m->loss);
+  };
+  if (8 * sm1 <= 200 * 1024)
+    loss(k_loss<8>, 8);
+  else
+    loss(k_loss<1>, 1);
   if ((st = mlp_check(m, "mlp loss")) != GW_OK) return st;
-  for (int l = m->nlayers - 1; l >= 0; --l) {
-    const int d = m->dout[l], di = m->din[l];
-    const int64_t n = Bn * d;
-    k_act_back<<<(unsigned)((n + 255) / 256), 256, 0, m->stream>>>(m->dH, m->Z[l], Bn, d, l == m->nlayers - 1, m->dZ,
-                                                                   m->dZh, m->dZT);
-    if ((st = mlp_check(m, "mlp act back")) != GW_OK) return st;
-    // dW = dZ^T H_in : [d][di], K = batch
-    if ((st = gemm(m, m->dZT, m->HT[l], m->gW[l], d, di, (int)Bn)) != GW_OK) return st;
-    k_colsum<<<(d + 127) / 128, 128, 0, m->stream>>>(m->dZ, Bn, d, m->gb[l]);
-    if ((st = mlp_check(m, "mlp colsum")) != GW_OK) return st;
-    // dH_in = dZ W : [B][di], K = d
-    if (l > 0 && (st = gemm(m, m->dZh, m->WTh[l], m->dH, (int)Bn, di, d)) != GW_OK) return st;
+  for (int l = e; l > 0; --l) {  // dZ of the layer below = (dZ W) act'(Z)
+    GemmArgs g{m->dZh[l], m->WTh[l], (int)Bn, m->din[l], m->dout[l], nullptr, m->Z[l - 1], m->dZh[l - 1], m->dZT[l - 1],
+               m->dZ[l - 1], 0};
+    if ((st = gemm<EPI_BACK>(m, g)) != GW_OK) return st;
+  }
+  cudaFuncSetAttribute(k_gemm_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
+  const int64_t np = gw_mlp_num_params(m);
+  const int kpart = dw_part(Bn), splits = (int)((Bn + kpart - 1) / kpart);
+  for (int l0 = 0; l0 < L; l0 += kMaxLayers) {
+    const int n = std::min(kMaxLayers, L - l0);
+    GemmJobs J{};
+    GradJobs D{};
+    J.njobs = D.nlayers = n;
+    J.kpart = kpart;
+    J.stride = D.stride = np;
+    D.splits = splits;
+    D.batch = Bn;
+    for (int i = 0; i < n; ++i) {  // dW = dZ^T H_in : [dout][din], K = batch
+      const int l = l0 + i, d = m->dout[l], di = m->din[l];
+      D.w0[i] = m->gW[l] - m->grads;
+      J.job[i] = GemmArgs{m->dZT[l], m->HT[l], d, di, (int)Bn, nullptr, nullptr, nullptr, nullptr, m->part + D.w0[i], 0};
+      J.tile0[i + 1] = J.tile0[i] + (d / 128) * (di / GN);
+      D.dZ[i] = m->dZ[l];
+      D.nw[i] = d * di;
+      D.d[i] = d;
+      D.wblk[i] = (D.nw[i] + 1023) / 1024;
+      D.blk0[i + 1] = D.blk0[i] + D.wblk[i] + d / 32;
+    }
+    k_gemm_dw<<<dim3(J.tile0[n], splits), GEMM_THREADS, G_SMEM, m->stream>>>(J, m->err);
+    if ((st = mlp_check(m, "mlp gemm")) != GW_OK) return st;
+    k_grads<<<D.blk0[n], 1024, 0, m->stream>>>(D, m->part, m->grads);
+    if ((st = mlp_check(m, "mlp gradients")) != GW_OK) return st;
   }
   return GW_OK;
 }
@@ -399,16 +547,14 @@ gw_status gw_mlp_create(gw_mlp** out, int nin, int nh, int nhidden, int nout, ui
     const double sc = l < m->nlayers - 1 ? std::sqrt(2.0 / din) : 0.1 / std::sqrt((double)din);
     std::vector<float> w((size_t)dout * din);
     for (auto& x : w) x = (float)(normal() * sc);
-    float *W, *b, *mW, *vW, *mb, *vb, *gW, *gb;
+    float *W, *b, *mW, *vW, *mb, *vb;
     __half *Wh, *WTh;
     ok &= cudaMalloc((void**)&W, sizeof(float) * w.size()) == cudaSuccess;
     ok &= cudaMalloc((void**)&mW, sizeof(float) * w.size()) == cudaSuccess;
     ok &= cudaMalloc((void**)&vW, sizeof(float) * w.size()) == cudaSuccess;
-    ok &= cudaMalloc((void**)&gW, sizeof(float) * w.size()) == cudaSuccess;
     ok &= cudaMalloc((void**)&b, sizeof(float) * dout) == cudaSuccess;
     ok &= cudaMalloc((void**)&mb, sizeof(float) * dout) == cudaSuccess;
     ok &= cudaMalloc((void**)&vb, sizeof(float) * dout) == cudaSuccess;
-    ok &= cudaMalloc((void**)&gb, sizeof(float) * dout) == cudaSuccess;
     ok &= cudaMalloc((void**)&Wh, sizeof(__half) * w.size()) == cudaSuccess;
     ok &= cudaMalloc((void**)&WTh, sizeof(__half) * w.size()) == cudaSuccess;
     if (!ok) break;
@@ -424,10 +570,15 @@ gw_status gw_mlp_create(gw_mlp** out, int nin, int nh, int nhidden, int nout, ui
     m->vW.push_back(vW);
     m->mb.push_back(mb);
     m->vb.push_back(vb);
-    m->gW.push_back(gW);
-    m->gb.push_back(gb);
     m->Wh.push_back(Wh);
     m->WTh.push_back(WTh);
+  }
+  const size_t np = ok ? (size_t)gw_mlp_num_params(m) : 1;
+  ok &= cudaMalloc((void**)&m->grads, sizeof(float) * np) == cudaSuccess;
+  for (int l = 0, o = 0; ok && l < m->nlayers; ++l) {
+    m->gW.push_back(m->grads + o);
+    m->gb.push_back(m->grads + o + m->dout[l] * m->din[l]);
+    o += m->dout[l] * (m->din[l] + 1);
   }
   ok &= cudaMalloc((void**)&m->loss, sizeof(float)) == cudaSuccess;
   ok &= cudaMalloc((void**)&m->err, sizeof(int)) == cudaSuccess;
@@ -452,16 +603,14 @@ gw_status gw_mlp_destroy(gw_mlp* m) {
   auto fr = [](void* p) {
     if (p) cudaFree(p);
   };
-  for (auto* v : {&m->W, &m->b, &m->mW, &m->vW, &m->mb, &m->vb, &m->gW, &m->gb, &m->Z})
+  for (auto* v : {&m->W, &m->b, &m->mW, &m->vW, &m->mb, &m->vb, &m->Z, &m->dZ})
     for (float* p : *v) fr(p);
-  for (auto* v : {&m->Wh, &m->WTh, &m->Hh, &m->HT})
+  for (auto* v : {&m->Wh, &m->WTh, &m->Hh, &m->HT, &m->dZh, &m->dZT})
     for (__half* p : *v) fr(p);
+  fr(m->grads);
+  fr(m->part);
   fr(m->Xh);
   fr(m->out);
-  fr(m->dZ);
-  fr(m->dZh);
-  fr(m->dZT);
-  fr(m->dH);
   fr(m->loss);
   fr(m->err);
   delete m;
@@ -489,16 +638,8 @@ gw_status gw_mlp_loss_grad(gw_mlp* m, int64_t batch, const float* x, int nx, con
   if ((st = forward(m, batch, x)) != GW_OK) return st;
   if ((st = backward(m, batch, x, Acpe, nx)) != GW_OK) return st;
   if (loss) cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToDevice, m->stream);
-  if (grads) {
-    size_t off = 0;
-    for (int l = 0; l < m->nlayers; ++l) {
-      const size_t nw = (size_t)m->dout[l] * m->din[l];
-      cudaMemcpyAsync(grads + off, m->gW[l], sizeof(float) * nw, cudaMemcpyDeviceToDevice, m->stream);
-      off += nw;
-      cudaMemcpyAsync(grads + off, m->gb[l], sizeof(float) * m->dout[l], cudaMemcpyDeviceToDevice, m->stream);
-      off += m->dout[l];
-    }
-  }
+  if (grads)
+    cudaMemcpyAsync(grads, m->grads, sizeof(float) * gw_mlp_num_params(m), cudaMemcpyDeviceToDevice, m->stream);
   return mlp_check(m, "mlp loss_grad");
 }
 
