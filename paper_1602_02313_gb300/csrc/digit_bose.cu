@@ -258,6 +258,7 @@ struct BoseUnit {
 };
 
 struct OpBoseFwd {
+  static constexpr int LV = 7;
   struct Job {
     const unsigned char *A, *B;
     const int *ea, *eb;
@@ -293,6 +294,7 @@ struct OpBoseFwd {
 };
 
 struct OpBoseBwd {
+  static constexpr int LV = 7;
   struct Job {
     const unsigned char *A, *B;
     const int *ea, *eb;

@@ -11,8 +11,12 @@
 // |a b|). The blocks' levels are added up in 64-bit integers and become one double per element at
 // the end. What is lost is the rounding of each operand to 2^-56 of its row's largest value and the
 // levels above 6: smaller than the rounding errors an FP64 accumulation of the same sum makes (the
-// measured errors against 64-bit sums are below the CUDA-core kernels' over all tested sizes).
+// measured errors of P and Sigma^c against exact sums are below the CUDA-core kernels' over all tested sizes).
 // Rows that hold an infinity or a nan give nan.
+//
+// Short sums leave FP64 fewer roundings to make: of the digits' loss most is the first level left out (six products,
+// 2^-56 of the rows' largest values, in the root mean square), so such a GEMM keeps eight levels (34
+// products) and every bit of its integer sums.
 //
 // Tile 128 x 64: the seven levels of 64 columns take 448 of the 512 TMEM columns. A 128 x 64 x 16 MMA
 // takes 48 clocks (its operands' 6 KB at 128 bytes per clock of shared memory; 32 of arithmetic), so
@@ -32,8 +36,9 @@ using namespace tc;
 
 constexpr int XS_N = 7;                       // digits per operand
 constexpr int XK = 16;                        // K values per chunk: one MMA step
+constexpr int XL_MAX = 8;                     // levels a GEMM may keep (OP::LV: 7 or 8)
 constexpr int X_BLK = 12;                     // chunks per accumulation block (192 k)
-constexpr int XN = 64;                        // output columns per tile: 7 levels x 64 = 448 TMEM columns
+constexpr int XN = 64;                        // output columns per tile: 8 levels x 64 = 512 TMEM columns at most
 constexpr int XA_SL = 128 * 32, XB_SL = XN * 32;  // bytes of one digit of an operand chunk
 constexpr int XA_BYTES = XS_N * XA_SL, XB_BYTES = XS_N * XB_SL;
 constexpr int XST_BYTES = XA_BYTES + XB_BYTES;    // 42 KB per stage
@@ -150,9 +155,16 @@ __device__ __forceinline__ double fix_to_double(long long y, int e) {
   return __longlong_as_double((long long)(b | ((uint64_t)y & 0x8000000000000000ull)));
 }
 
+// (hi 2^32 + lo) 2^e with all of the sum's leading bits (|lo| < 2^61), where a fixed number of dropped bits, which
+// has to cover the largest sum that K allows, would cost a short or cancelling one its last bits
+__device__ __forceinline__ double fix_to_double(long long hi, long long lo, int e) {
+  const int s = max(0, 34 - __clzll(hi ^ (hi >> 63)));
+  return fix_to_double((hi << (32 - s)) + (lo >> s), e + s);
+}
+
 // ------------------------------------------------------------------ the digit GEMM
 struct XSmem {
-  uint64_t full[X_ST], empty[X_ST], done, lvl[XS_N], fin, never;
+  uint64_t full[X_ST], empty[X_ST], done, lvl[XL_MAX], fin, never;
   uint32_t tslot;
   int abort_flag, no_dealloc;
   double red[3][128];
@@ -161,6 +173,7 @@ struct XSmem {
 // The GEMM C = A B^T of digit images, one persistent kernel; what a unit is and what becomes of its tiles
 // is an OP class:
 //   OP::Job  kernel parameters (with sh, the bits of the 96-bit sums dropped at the end: drop_bits)
+//   OP::LV   levels kept: 7, or 8 with tile(J, U, n, hi, lo), the elements being (hi 2^32 + lo) 2^(ea + eb - 62)
 //   OP::Unit (J, u): n0, n1 (the tiles n of the unit, one after another), A(J, n), B(J, n) (operand images,
 //            chunks XA_BYTES / XB_BYTES apart), range(J, n, c0, c1) (the chunks of tile n)
 //   OP(J, U, r, part): the epilogue thread of row r (0 .. 127) and columns 16 part .. + 15 of the unit's tiles;
@@ -180,7 +193,7 @@ __global__ void __launch_bounds__(X_THREADS, 1)
       mbar_init(&S.empty[s], 1);
     }
     mbar_init(&S.done, 1);
-    for (int s = 0; s < XS_N; ++s) mbar_init(&S.lvl[s], X_EPI);
+    for (int s = 0; s < OP::LV; ++s) mbar_init(&S.lvl[s], X_EPI);
     mbar_init(&S.fin, 1);
     mbar_init(&S.never, 1);
     S.abort_flag = 0;
@@ -247,7 +260,7 @@ __global__ void __launch_bounds__(X_THREADS, 1)
             const uint32_t a = a0 + s * (XST_BYTES >> 4), b = b0 + s * (XST_BYTES >> 4);
             if (c == cb) {
 #pragma unroll
-              for (int l = 0; l < XS_N; ++l) {
+              for (int l = 0; l < OP::LV; ++l) {
                 // the previous block's level l has been read (its first MMA overwrites it)
                 if (blk > 0) {
                   live = live && __all_sync(0xffffffffu, wait_bar(&S.lvl[l], (blk - 1) & 1, &S.abort_flag, err, wait_cycles));
@@ -255,17 +268,18 @@ __global__ void __launch_bounds__(X_THREADS, 1)
                 }
                 if (lead) {
 #pragma unroll
-                  for (int x = 0; x <= l; ++x)
-                    mma_f16_lo(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, x > 0);
+                  for (int x = l < XS_N ? 0 : l - XS_N + 1; x <= l && x < XS_N; ++x)
+                    mma_f16_lo(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id,
+                               x > (l < XS_N ? 0 : l - XS_N + 1));
                 }
                 __syncwarp();
               }
             } else {
               if (lead) {
 #pragma unroll
-                for (int l = 0; l < XS_N; ++l)
+                for (int l = 0; l < OP::LV; ++l)
 #pragma unroll
-                  for (int x = 0; x <= l; ++x)
+                  for (int x = l < XS_N ? 0 : l - XS_N + 1; x <= l && x < XS_N; ++x)
                     mma_f16_lo(tbase + XN * l, a + x * (XA_SL >> 4), b + (l - x) * (XB_SL >> 4), dh, id, 1);
               }
             }
@@ -307,8 +321,8 @@ __global__ void __launch_bounds__(X_THREADS, 1)
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
-          for (int l = 0; l < XS_N; ++l) {
-            constexpr int kShift[XS_N] = {16, 8, 0, 24, 16, 8, 0};
+          for (int l = 0; l < OP::LV; ++l) {
+            constexpr int kShift[XL_MAX] = {16, 8, 0, 24, 16, 8, 0, 0};
             float v[16];
             tmem_ld16(tw + XN * l, v);
             tc_fence_before();
@@ -316,16 +330,20 @@ __global__ void __launch_bounds__(X_THREADS, 1)
             if (lane == 0) mbar_arrive(&S.lvl[l]);  // the next block may overwrite this level
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
-              const long long t = (long long)__float2int_rn(v[e]) * (1 << kShift[l]);
+              const long long t = (long long)__float2int_rn(l < XS_N ? v[e] : v[e] * 0.00390625f) * (1 << kShift[l]);
               if (l < 3) hi[e] += t; else lo[e] += t;
             }
           }
         }
         if (!ok) break;
         // element = (hi 2^32 + lo) 2^(ea + eb - 62) = y 2^(ea + eb - 62 + sh), |y| < 2^63
+        if constexpr (OP::LV == XL_MAX) {
+          op.tile(J, U, n, hi, lo);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) hi[e] = (hi[e] << (32 - J.sh)) + (lo[e] >> J.sh);
-        op.tile(J, U, n, hi);
+          for (int e = 0; e < 16; ++e) hi[e] = (hi[e] << (32 - J.sh)) + (lo[e] >> J.sh);
+          op.tile(J, U, n, hi);
+        }
       }
       op.finish(J, U, S.red, ok);
     }

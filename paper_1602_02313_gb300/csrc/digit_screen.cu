@@ -272,6 +272,7 @@ __global__ void __launch_bounds__(256) k_gj_cols(GjJob J) {
 
 // GEMM 1: unit = (system, M tile of columns c), tiles n over the 2 bw columns (Re, Im of row r)
 struct OpGjRows {
+  static constexpr int LV = 7;
   using Job = GjJob;
   struct Unit {
     int s, m, n0, n1;
@@ -307,6 +308,7 @@ struct OpGjRows {
 
 // GEMM 2: unit = (system, M tile of rows i, N tile of 32 columns c)
 struct OpGjUpdate {
+  static constexpr int LV = 7;
   using Job = GjJob;
   struct Unit {
     int s, m, n0, n1;

@@ -20,6 +20,7 @@ namespace {
 // ------------------------------------------------------------------ what the GEMM does with its tiles
 // Polarization: unit = (K split, M tile, N tile), C[split][row][n] = sum over the split's chunks.
 struct OpStore {
+  static constexpr int LV = 7;
   struct Job {
     const unsigned char *A, *B;  // [M tile][chunk], [N tile][chunk]
     const int *ea, *eb;          // row exponents [rows], [ncols]
@@ -53,6 +54,7 @@ struct OpStore {
 // Self-energy: unit = (M tile, tau), all N tiles jt (32 columns J of Y1 beside the same J of Y2) over the
 // K chunks I <= J, dotted with M: D[row][tau].
 struct OpDot {
+  static constexpr int LV = 7;
   struct Job {
     const unsigned char *A, *B;  // [M tile][chunk], [tau][N tile][chunk]
     const int *ea, *eb;          // row exponents [rows], [tau][J]

@@ -152,6 +152,8 @@ gw_status launch_pol_fp64(gw_ctx* c, int iq, const double* G, double* P);
 // FP64 on the tensor cores (exact digit products); GW_EUNSUPPORTED when the digit workspace cannot be had
 gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P);
 gw_status launch_sigma_exact(gw_ctx* c, int iq, const double* G, const double* W, double* S);
+gw_status launch_offdiag_digits(gw_ctx* c, int iq, const double* G, const double* occ, const double* W, double* S,
+                                double* Sx);
 // W~ by digit products; aug: at least one matrix [ni][ni] per system; GW_EUNSUPPORTED as above
 gw_status launch_screen_digits(gw_ctx* c, int iq0, int nqb, const double* P, double* W, int* info, double* aug);
 gw_status bose_digits(gw_ctx* c);  // at gw_create, after the transform matrices
