@@ -265,7 +265,7 @@ gw_status gw_selfenergy_offdiag(gw_ctx* ctx, int iq, const double* G_tau, const 
  * did not reach 1e-15 relative off-diagonal norm in 40 sweeps (G is still written), or 2 + j
  * for a zero pivot at elimination step j of some frequency (that k's G and occ not written).
  * FP64 on the CUDA cores; nb <= 256 (else GW_EINVAL); workspace
- * ~ nk nb^2 (4 nw + 2) 16 bytes, grown on use. */
+ * ~ nk nb^2 (3 nw + 2) 16 bytes (4 nw + 2 above nb 113), grown on use. */
 gw_status gw_dyson_matrix(gw_ctx* ctx, const double* eps, const double* Sx, const double* vxc, const double* Sc_tau,
                           double* G_tau, double* occ, int* info);
 

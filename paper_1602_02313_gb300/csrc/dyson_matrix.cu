@@ -24,6 +24,9 @@ namespace {
 
 constexpr int kDmThreads = 256;
 constexpr int kDmMaxSweeps = 40;
+// k_dm_inv keeps its matrix in shared memory up to this: 1014 -> 194 us at Nk 8, Nb 32, 16 w, against the augmented
+// matrix in the workspace with a serial pivot search; above it the same elimination runs on the workspace.
+constexpr size_t kDmSmem = 200 * 1024;
 
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
@@ -209,9 +212,13 @@ __global__ void __launch_bounds__(kDmThreads) k_dm_eig(const double* __restrict_
   if (t == 0) info[k] = stop_flag ? 0 : 1;
 }
 
-// One block per (k, w): Gauss-Jordan inversion with partial pivoting of B = i w - H~ - Sigma^c(i w)
-// on the augmented [B | 1] (workspace [nb][2 nb]), then the remainder R = B^-1 - U (i w - lambda)^-1 U^+
-// as the transforms of the real tau-functions Re G and Im G: ah = (R + R^T) / 2, bh = (R - R^T) / 2i.
+// One block per (k, w): Gauss-Jordan inversion with partial pivoting of B = i w - H~ - Sigma^c(i w), in place
+// (column col of the inverse under construction takes the place of the column just eliminated; who[] undoes the
+// row exchanges at the end), then the remainder R = B^-1 - U (i w - lambda)^-1 U^+ as the transforms of the real
+// tau-functions Re G and Im G: ah = (R + R^T) / 2 (symmetric), bh = (R - R^T) / 2i (antisymmetric), formed once
+// for n <= m. The matrix is in shared memory up to 200 KiB (nb <= 113), in the workspace above. Bound by the FP64
+// pipe (6 nb^3 + 4 nb^3 operations per block) and the chain of nb pivots. Measured at Nk 8, Nb 32, 16 w: see kDmSmem.
+template <bool SM>
 __global__ void __launch_bounds__(kDmThreads) k_dm_inv(const double* __restrict__ eps, const double2* __restrict__ Sx,
                                                        const double2* __restrict__ vxc, const double2* __restrict__ Siw,
                                                        const int* __restrict__ widx, double beta, int nb, int nbp,
@@ -219,108 +226,119 @@ __global__ void __launch_bounds__(kDmThreads) k_dm_inv(const double* __restrict_
                                                        const double* __restrict__ lam, double2* __restrict__ aug,
                                                        double2* __restrict__ ah, double2* __restrict__ bh,
                                                        int* __restrict__ info) {
-  __shared__ double pv[kDmThreads];
-  __shared__ int pi[kDmThreads];
-  __shared__ int piv_row, fail;
-  const int k = blockIdx.x / nw, j = blockIdx.x % nw, t = threadIdx.x;
+  extern __shared__ double2 xs[];
+  __shared__ double2 prow[256], orow[256], fcol[256], inv_p;  // pivot row / p, the row it changes places with, column col
+  __shared__ int who[256], pos[256], piv_row, fail;
+  const int k = blockIdx.x / nw, j = blockIdx.x % nw, t = threadIdx.x, tx = t & 31, ty = t >> 5;
   const double w = (2.0 * widx[j] + 1.0) * M_PI / beta;
-  const int n2 = 2 * nb;
-  double2* X = aug + (size_t)blockIdx.x * nb * n2;
-  for (int e = t; e < nb * n2; e += kDmThreads) {
-    const int r = e / n2, c = e % n2;
-    double2 v = make_double2(0.0, 0.0);
-    if (c < nb) {
+  const int ld = nb | 1;  // odd: the pivot search reads a column without bank conflicts
+  double2* X = SM ? xs : aug + (size_t)blockIdx.x * nb * ld;
+  for (int r = ty; r < nb; r += kDmThreads / 32)
+    for (int c = tx; c < nb; c += 32) {
       const size_t o = ((size_t)k * nb + r) * nb + c;
       const double2 h = csub(Sx ? Sx[o] : make_double2(0.0, 0.0), vxc ? vxc[o] : make_double2(0.0, 0.0));
       const double2 s = Siw ? Siw[o * nw + j] : make_double2(0.0, 0.0);
-      v = make_double2(-h.x - s.x, -h.y - s.y);
+      double2 v = make_double2(-h.x - s.x, -h.y - s.y);
       if (r == c) {
         v.x -= eps[(size_t)k * nb + r];
         v.y += w;
       }
-    } else if (c - nb == r) {
-      v.x = 1.0;
+      X[r * ld + c] = v;
     }
-    X[e] = v;
-  }
+  for (int r = t; r < nb; r += kDmThreads) who[r] = r;
   if (t == 0) fail = 0;
   __syncthreads();
   for (int col = 0; col < nb; ++col) {
-    // pivot: largest |.| in column col among rows >= col (first on ties)
-    double best = -1.0;
-    int br = col;
-    for (int r = col + t; r < nb; r += kDmThreads) {
-      const double2 v = X[(size_t)r * n2 + col];
-      const double m = v.x * v.x + v.y * v.y;
-      if (m > best) {
-        best = m;
-        br = r;
-      }
-    }
-    pv[t] = best;
-    pi[t] = br;
-    __syncthreads();
-    if (t == 0) {
-      double b = -1.0;
-      int r0 = col;
-      for (int i = 0; i < kDmThreads; ++i)
-        if (pv[i] > b || (pv[i] == b && pi[i] < r0)) {
-          b = pv[i];
-          r0 = pi[i];
+    if (ty == 0) {
+      // pivot: largest |.| in column col among rows >= col (first on ties)
+      double best = -1.0;
+      int br = col;
+      for (int r = col + tx; r < nb; r += 32) {
+        const double2 v = X[r * ld + col];
+        const double m = v.x * v.x + v.y * v.y;
+        if (m > best) {
+          best = m;
+          br = r;
         }
-      piv_row = r0;
-      if (!(b > 0.0) && !fail) {
-        fail = 1;
-        atomicMax(info + k, 2 + col);
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        const double b2 = __shfl_xor_sync(0xffffffffu, best, o);
+        const int r2 = __shfl_xor_sync(0xffffffffu, br, o);
+        if (b2 > best || (b2 == best && r2 < br)) {
+          best = b2;
+          br = r2;
+        }
+      }
+      if (tx == 0) {
+        piv_row = br;
+        inv_p = cinv(X[br * ld + col]);
+        const int a = who[col];
+        who[col] = who[br];
+        who[br] = a;
+        if (!(best > 0.0)) {
+          fail = 1;
+          atomicMax(info + k, 2 + col);
+        }
       }
     }
     __syncthreads();
     if (fail) return;  // uniform: the block stops, its output is not written
     const int pr = piv_row;
-    if (pr != col)
-      for (int c = t; c < n2; c += kDmThreads) {
-        const double2 a = X[(size_t)col * n2 + c];
-        X[(size_t)col * n2 + c] = X[(size_t)pr * n2 + c];
-        X[(size_t)pr * n2 + c] = a;
-      }
-    __syncthreads();
-    const double2 inv = cinv(X[(size_t)col * n2 + col]);
-    __syncthreads();
-    for (int c = t; c < n2; c += kDmThreads) X[(size_t)col * n2 + c] = cmul(X[(size_t)col * n2 + c], inv);
-    __syncthreads();
-    for (int e = t; e < nb * n2; e += kDmThreads) {
-      const int r = e / n2, c = e % n2;
-      if (r == col) continue;
-      const double2 f = X[(size_t)r * n2 + col];
-      if (c == col) continue;
-      X[e] = csub(X[e], cmul(f, X[(size_t)col * n2 + c]));
+    const double2 inv = inv_p;
+    for (int c = t; c < nb; c += kDmThreads) {
+      prow[c] = c == col ? inv : cmul(X[pr * ld + c], inv);
+      orow[c] = X[col * ld + c];
+      fcol[c] = c == pr ? X[col * ld + col] : X[c * ld + col];
     }
     __syncthreads();
-    for (int r = t; r < nb; r += kDmThreads)
-      if (r != col) X[(size_t)r * n2 + col] = make_double2(0.0, 0.0);
+    for (int r = ty; r < nb; r += kDmThreads / 32) {
+      const double2 f = fcol[r];
+      for (int c = tx; c < nb; c += 32) {
+        const double2 p = prow[c];
+        if (r == col) {
+          X[r * ld + c] = p;
+        } else {
+          const double2 x = c == col ? make_double2(0.0, 0.0) : r == pr ? orow[c] : X[r * ld + c];
+          X[r * ld + c] = csub(x, cmul(f, p));
+        }
+      }
+    }
     __syncthreads();
   }
-  // R = B^-1 - U diag(1 / (i w - lambda)) U^+, split into the two real-function transforms
+  // column c of X is column who[c] of the inverse
   const double2* U = Uw + (size_t)k * nbp * nbp;
   const double* lk = lam + (size_t)k * nbp;
-  __shared__ double2 gl[256];
-  for (int a = t; a < nbp; a += kDmThreads) gl[a] = cinv(make_double2(-lk[a], w));  // 1 / (i w - lambda_a)
+  for (int c = t; c < nb; c += kDmThreads) pos[who[c]] = c;
+  for (int a = t; a < nbp; a += kDmThreads) prow[a] = cinv(make_double2(-lk[a], w));  // 1 / (i w - lambda_a)
   __syncthreads();
-  for (int e = t; e < nb * nb; e += kDmThreads) {
-    const int n = e / nb, m = e % nb;
-    double2 rnm = X[(size_t)n * n2 + nb + m], rmn = X[(size_t)m * n2 + nb + n];
+  // n <= m: rows f and nb - 1 - f of the upper triangle make nb + 1 elements together
+  for (int e = t; e < (nb + 1) / 2 * (nb + 1); e += kDmThreads) {
+    const int f = e / (nb + 1), i = e - f * (nb + 1);
+    const bool second = i >= nb - f;
+    const int n = second ? nb - 1 - f : f, m = second ? n + i - (nb - f) : f + i;
+    if (second && n == f) continue;  // the middle row of an odd nb stands alone
+    double s1 = 0.0, s2 = 0.0, s3 = 0.0, s4 = 0.0;
     for (int a = 0; a < nbp; ++a) {
-      const double2 g = gl[a];
-      const double2 un = U[(size_t)n * nbp + a], um = U[(size_t)m * nbp + a];
-      // (U g U^+)_nm = un g conj(um), (U g U^+)_mn = um g conj(un)
-      const double2 x = cmul(un, make_double2(um.x, -um.y)), y = cmul(um, make_double2(un.x, -un.y));
-      rnm = csub(rnm, cmul(g, x));
-      rmn = csub(rmn, cmul(g, y));
+      const double2 g = prow[a], un = U[(size_t)n * nbp + a], um = U[(size_t)m * nbp + a];
+      const double xr = fma(un.x, um.x, un.y * um.y), xi = fma(un.y, um.x, -(un.x * um.y));  // un conj(um)
+      s1 = fma(g.x, xr, s1);
+      s2 = fma(g.y, xr, s2);
+      s3 = fma(g.y, xi, s3);
+      s4 = fma(g.x, xi, s4);
     }
+    // sum_a un g conj(um) = (s1 - s3, s2 + s4), sum_a um g conj(un) = (s1 + s3, s2 - s4)
+    const double2 rnm = X[n * ld + pos[m]], rmn = X[m * ld + pos[n]];
+    const double2 a = make_double2(0.5 * (rnm.x + rmn.x) - s1, 0.5 * (rnm.y + rmn.y) - s2);
+    const double2 b = make_double2(0.5 * (rnm.y - rmn.y) - s4, -0.5 * (rnm.x - rmn.x) - s3);  // -i (R_nm - R_mn) / 2
     const size_t o = (((size_t)k * nb + n) * nb + m) * nw + j;
-    ah[o] = make_double2(0.5 * (rnm.x + rmn.x), 0.5 * (rnm.y + rmn.y));
-    const double2 d = csub(rnm, rmn);  // (R_nm - R_mn) / (2 i) = -i d / 2
-    bh[o] = make_double2(0.5 * d.y, -0.5 * d.x);
+    ah[o] = a;
+    bh[o] = b;
+    if (n != m) {
+      const size_t q = (((size_t)k * nb + m) * nb + n) * nw + j;
+      ah[q] = a;
+      bh[q] = make_double2(-b.x, -b.y);
+    }
   }
 }
 
@@ -388,7 +406,9 @@ extern "C" gw_status gw_dyson_matrix(gw_ctx* c, const double* eps, const double*
   const size_t el = (size_t)nk * nb * nb;
   const size_t b_siw = Sc_tau ? el * nw * sizeof(double2) : 0;
   const size_t b_eig = 2 * (size_t)nk * nbp * nbp * sizeof(double2) + (size_t)nk * nbp * sizeof(double);
-  const size_t b_aug = (size_t)nk * nw * nb * 2 * nb * sizeof(double2);
+  const size_t x_sm = (size_t)nb * (nb | 1) * sizeof(double2);  // one matrix of k_dm_inv
+  const bool sm = x_sm <= kDmSmem;
+  const size_t b_aug = sm ? 0 : (size_t)nk * nw * x_sm;
   const size_t b_hat = 2 * el * nw * sizeof(double2);
   const size_t b_g0 = (size_t)nk * nbp * (nt + 1) * sizeof(double);
   const size_t need = b_siw + b_eig + b_aug + b_hat + b_g0 + 1024;
@@ -410,7 +430,7 @@ extern "C" gw_status gw_dyson_matrix(gw_ctx* c, const double* eps, const double*
   double* lam = (double*)(U + (size_t)nk * nbp * nbp);
   w += b_eig;
   double2* aug = (double2*)(((uintptr_t)w + 255) & ~(uintptr_t)255);
-  double2* ah = aug + (size_t)nk * nw * nb * 2 * nb;
+  double2* ah = aug + b_aug / sizeof(double2);
   double2* bh = ah + el * nw;
   double* g0t = (double*)(bh + el * nw);
   gw_status st;
@@ -423,9 +443,11 @@ extern "C" gw_status gw_dyson_matrix(gw_ctx* c, const double* eps, const double*
   k_dm_eig<<<(unsigned)nk, kDmThreads, 0, c->stream>>>(eps, (const double2*)Sx, (const double2*)vxc, nb, nbp, A, U,
                                                        lam, info);
   if ((st = check_launch(c, "dm_eig")) != GW_OK) return st;
-  k_dm_inv<<<(unsigned)(nk * nw), kDmThreads, 0, c->stream>>>(eps, (const double2*)Sx, (const double2*)vxc, Siw,
-                                                              c->d_widx, c->beta, nb, nbp, nw, U, lam, aug, ah, bh,
-                                                              info);
+  auto inv = sm ? k_dm_inv<true> : k_dm_inv<false>;
+  if (sm) cudaFuncSetAttribute(inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)x_sm);
+  inv<<<(unsigned)(nk * nw), kDmThreads, sm ? x_sm : 0, c->stream>>>(eps, (const double2*)Sx, (const double2*)vxc, Siw,
+                                                                    c->d_widx, c->beta, nb, nbp, nw, U, lam, aug, ah,
+                                                                    bh, info);
   if ((st = check_launch(c, "dm_inv")) != GW_OK) return st;
   const int64_t ng = (int64_t)nk * nbp * (nt + 1);
   k_dm_g0tab<<<(unsigned)((ng + 255) / 256), 256, 0, c->stream>>>(lam, c->d_tau, c->beta, nk, nbp, nt, g0t);
