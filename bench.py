@@ -486,26 +486,30 @@ def run_offdiag(args):
     for _ in range(args.warmup):
         ctx.selfenergy_offdiag(0, G, occ, W, S, Sx)
     torch.cuda.synchronize()
+    launches0 = ctx.launch_count()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record(st)
     for _ in range(args.steps):
         ctx.selfenergy_offdiag(0, G, occ, W, S, Sx)
     e1.record(st)
     torch.cuda.synchronize()
+    launches = ctx.launch_count() - launches0
     ms = e0.elapsed_time(e1) / args.steps
     nk, nb, ni, nt = cr.nk, cr.nb, cr.ni, gr.ntau
     macs = float(nk) * nt * nb * (ni * ni * nb + ni * nb * nb) + float(nk) * nb ** 3 * ni
-    fp64_tf, _ = gw.measure_alu(0)
+    # each product is 34 products of 8-bit digits on the tensor cores
+    peaks = _peaks()
+    peak = peaks["tensor_sustained"] / 34.0
     ach = 8.0 * macs / (ms * 1e-3) / 1e12
     out = {"metric": "off-diagonal self-energy time, one q (Eqs. sigc, sigx as band matrices)", "value": ms,
            "unit": "ms", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
            "higher_is_better": False, "scaling": "strong", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
            "config": {"workload": f"one q: Nk={nk}, Nb={nb}, NI={ni}, Ntau={nt}"},
-           "gpu_launches": 2 * args.steps,
-           "roofline_alu": {"bound": "alu", "kernel": "k_sigma_offdiag + k_sigx_offdiag", "achieved": ach,
-                            "peak": fp64_tf, "unit": "TFLOP/s FP64", "frac": ach / fp64_tf,
-                            "peak_source": "measured FP64 FMA rate of this GPU (gw_measure_alu, this run)"},
-           "roofline": None, "cpu_baseline": None, "e2e": None}
+           "gpu_launches": int(launches), "roofline_alu": None,
+           "roofline": {"bound": "tensor", "kernel": "gw_selfenergy_offdiag (whole call, digit products)",
+                        "achieved": ach, "peak": peak, "unit": "TFLOP/s FP64", "frac": ach / peak,
+                        "peak_source": peaks["source"] + ", sustained bf16/fp16 dense / 34 digit products"},
+           "cpu_baseline": None, "e2e": None}
     print(json.dumps(out))
     ctx.close()
 
@@ -977,21 +981,21 @@ def main():
         kname = dom
         achieved = per_launch_flops[dom] / (kt[dom] * 1e-3) / 1e12 if dom in kt else None
         label = "gw_" + dom + " (whole call)"
-    # the screening against the measured rate of the FP32 pipes: NI^3 complex multiply-adds per
-    # (q, nu) system (in-place Gauss-Jordan inverse); a float-float complex multiply-add is 48
-    # FP32-pipe operations, an FP32 one 4 FMAs
+    # the screening: NI^3 complex multiply-adds per (q, nu) system (in-place Gauss-Jordan inverse). FP32:
+    # against the measured rate of the FP32 pipes, 4 FMAs each. GW_F32X2: digit products on the tensor
+    # cores, 8 x 28 flops each, against their sustained rate (the event pair brackets all launches of a call)
     roof_alu = None
     if "k_screen_inv" in kern and prec != gw.GW_FP64:
         fp64_tf, fp32_tf = gw.measure_alu(local)
         macs = float(cr.ni) ** 3 * len(chain.iqs) * len(gr.nu_idx) * args.steps
         ach = macs / (kern["k_screen_inv"]["total_ms"] * 1e-3) / 1e9
-        ops = 48.0 if args.screen == "f32x2" else 4.0
-        arith_name = "float-float" if args.screen == "f32x2" else "FP32"
-        peak_ff = fp32_tf * 1e3 / (2.0 * ops)  # 2 flops per FP32-pipe operation
-        roof_alu = {"bound": "alu", "kernel": f"k_screen_inv<{arith_name}> (CUDA events around each launch)",
-                    "achieved": ach, "peak": peak_ff, "unit": f"G complex {arith_name} MAC/s", "frac": ach / peak_ff,
-                    "peak_source": f"measured FP32 FMA rate of this GPU (gw_measure_alu, this run) / {ops:.0f} "
-                                   f"operations per {arith_name} complex multiply-add",
+        digits = args.screen == "f32x2"
+        peak_mac = peaks["tensor_sustained"] * 1e3 / 224.0 if digits else fp32_tf * 1e3 / 8.0
+        roof_alu = {"bound": "tensor" if digits else "alu",
+                    "kernel": "gw_screen (GW_F32X2, digit products)" if digits else "k_screen_inv<FP32>",
+                    "achieved": ach, "peak": peak_mac, "unit": "G complex MAC/s", "frac": ach / peak_mac,
+                    "peak_source": peaks["source"] + ", sustained bf16/fp16 dense / (8 x 28) flops per complex MAC"
+                    if digits else "measured FP32 FMA rate of this GPU (gw_measure_alu, this run) / 4 FMAs per complex MAC",
                     "measured_fp64_tflops": fp64_tf, "measured_fp32_tflops": fp32_tf}
     roof = {"bound": "tensor" if prec != gw.GW_FP64 else "alu", "kernel": label,
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
