@@ -204,9 +204,9 @@ def _dtype(args):
     """The arithmetic of each step of the benchmarked chain."""
     if args.prec == "fp64":
         return "f64 (every step)"
-    scr = "f32x2 (float-float)" if args.screen == "f32x2" else "f32"
+    scr = "f32x2 (exact digit products on tensor cores, f64 matrix)" if args.screen == "f32x2" else "f32"
     return (f"P and Sigma^c: fp16x2 split on tensor cores, fp32 accumulation, f32x2 segment sums; "
-            f"dielectric solve: {scr}; bosonic transforms and Sigma^x: f32x2 (float-float); "
+            f"dielectric solve: {scr}; bosonic transforms: exact digit products; Sigma^x: f32x2 (float-float); "
             f"G, Dyson, fermionic transforms, continuation: f64")
 
 
@@ -955,7 +955,7 @@ def main():
     ctx.kernel_timing(False)
     per_launch_flops = {"polarization": fp, "selfenergy": fs, "k_pol_tc": fp, "k_sig_tc": fs}
     # tensor-core MMA flops per algorithmic flop: 3 split products times the cover of P's strips;
-    # Sigma runs 4 real GEMMs over the upper triangle of W~, (nkc + 1) / (2 nkc) of the columns,
+    # Sigma runs 4 real GEMMs over the upper triangle of W~ in 16-row steps, (nkc + 1) / (2 nkc) of the columns,
     # against 4 NI^2 MACs counted
     ni_ = cr.ni
     # P up to NI = 256: E = Re P + Im P in strips of 128 rows over all NI columns (rows padded to
@@ -964,7 +964,7 @@ def main():
         strip_cover = 128 * ((ni_ + 127) // 128) / float(ni_)
     else:
         strip_cover = sum(128 * (ni_ - 128 * i) for i in range((ni_ + 127) // 128)) / (ni_ * ni_ / 2.0)
-    nkc_ = ni_ // 32
+    nkc_ = ni_ // 16
     mma_factor = {"k_pol_tc": 3.0 * strip_cover, "k_sig_tc": 3.0 * (nkc_ + 1) / (2.0 * nkc_)}
     peaks = _peaks()
     peak = peaks["tensor_sustained"]
