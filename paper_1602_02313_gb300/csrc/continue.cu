@@ -156,8 +156,6 @@ __global__ void k_pade(int64_t nprob, const double2* __restrict__ sig, int ncont
 constexpr int kCpeMaxGrid = 128;
 constexpr int kSlots = kCpeMaxGrid / 32;
 constexpr double kSeedSupport = 1e-2;  // seed weights above this fraction of the largest start active
-constexpr int kNnlsRows = 64;          // rows of the factor a first launch over many problems keeps (see the launch)
-constexpr int kNnlsRedo = -1;          // info of a problem whose passive set outgrew them
 constexpr int kWarmSolves = 8;         // solves allowed to turn the seed's support into a feasible point
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -200,22 +198,13 @@ __device__ bool chol_append(const NnlsWarp& S, const double* __restrict__ N, int
   for (int sk = 0; sk < kSlots; ++sk) {
     if (32 * sk >= p) break;
     const int kend = min(32, p - 32 * sk);
-    // column k + 1 of L is loaded while column k is used: what is serial is a shuffle, a product and an fma
-    double dk = S.dinv[32 * sk], c[kSlots];
-#pragma unroll
-    for (int s = sk; s < kSlots; ++s) {
-      const int i = lane + 32 * s;
-      c[s] = i > 32 * sk && i < p ? S.L[tri(i) + 32 * sk] : 0.0;
-    }
     for (int kk = 0; kk < kend; ++kk) {
-      const int k = 32 * sk + kk, kn = 32 * sk + min(kk + 1, kend - 1);
-      const double lk = __shfl_sync(0xffffffffu, r[sk], kk) * dk;
-      dk = S.dinv[kn];
+      const int k = 32 * sk + kk;
+      const double lk = __shfl_sync(0xffffffffu, r[sk], kk) * S.dinv[k];
 #pragma unroll
       for (int s = sk; s < kSlots; ++s) {
         const int i = lane + 32 * s;
-        if (i > k && i < p) r[s] = fma(-c[s], lk, r[s]);
-        if (i > kn && i < p) c[s] = S.L[tri(i) + kn];
+        if (i > k && i < p) r[s] = fma(-S.L[tri(i) + k], lk, r[s]);
       }
     }
   }
@@ -257,22 +246,14 @@ __device__ void chol_solve(const NnlsWarp& S, int p, const double (&yv)[kSlots],
 #pragma unroll
   for (int sk = kSlots - 1; sk >= 0; --sk) {
     if (32 * sk >= p) continue;
-    const int kend = min(32, p - 32 * sk), k1 = 32 * sk + kend - 1;
-    double dk = S.dinv[k1], c[kSlots];  // row k - 1 of L is loaded while row k is used
-#pragma unroll
-    for (int s = 0; s <= sk; ++s) {
-      const int j = lane + 32 * s;
-      c[s] = j < k1 ? S.L[tri(k1) + j] : 0.0;
-    }
+    const int kend = min(32, p - 32 * sk);
     for (int kk = kend - 1; kk >= 0; --kk) {
-      const int k = 32 * sk + kk, kn = 32 * sk + max(kk - 1, 0);
-      const double zk = __shfl_sync(0xffffffffu, t[sk], kk) * dk;
-      dk = S.dinv[kn];
+      const int k = 32 * sk + kk;
+      const double zk = __shfl_sync(0xffffffffu, t[sk], kk) * S.dinv[k];
 #pragma unroll
       for (int s = 0; s <= sk; ++s) {
         const int j = lane + 32 * s;
-        if (j < k) t[s] = fma(-c[s], zk, t[s]);
-        if (j < kn) c[s] = S.L[tri(kn) + j];
+        if (j < k) t[s] = fma(-S.L[tri(k) + j], zk, t[s]);
       }
     }
   }
@@ -322,12 +303,11 @@ __device__ int chol_remove(const NnlsWarp& S, const double* __restrict__ N, int 
 __global__ void __launch_bounds__(32) k_cpe_nnls(int64_t nprob, const double2* __restrict__ sig, int ncont,
                                                  const double* __restrict__ A, const double* __restrict__ N, int ng,
                                                  const double* __restrict__ b0, double* __restrict__ bout,
-                                                 int* __restrict__ info, int* __restrict__ iters, int cap, int redo) {
+                                                 int* __restrict__ info, int* __restrict__ iters) {
   extern __shared__ double sm[];
-  if (redo && info[blockIdx.x] != kNnlsRedo) return;
   NnlsWarp S;
   S.L = sm;
-  S.dinv = S.L + tri(cap);
+  S.dinv = S.L + tri(ng);
   S.cv = S.dinv + kCpeMaxGrid;
   S.xv = S.cv + kCpeMaxGrid;
   S.zv = S.xv + kCpeMaxGrid;
@@ -377,10 +357,6 @@ __global__ void __launch_bounds__(32) k_cpe_nnls(int64_t nprob, const double2* _
       nsel += __popc(bal);
     }
     __syncwarp();
-    if (nsel > cap) {
-      if (lane == 0) info[prob] = kNnlsRedo;
-      return;
-    }
     for (int q = 0; q < nsel; ++q)
       if (chol_append(S, N, ng, p, S.lst[q], yv, lane)) ++p;
     if (p > 0) {
@@ -394,7 +370,6 @@ __global__ void __launch_bounds__(32) k_cpe_nnls(int64_t nprob, const double2* _
       double w[kSlots];
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) w[s] = S.cv[lane + 32 * s];
-#pragma unroll 4
       for (int k = 0; k < p; ++k) {
         const int mk = S.idx[k];
         const double xk = S.xv[mk];
@@ -427,10 +402,6 @@ __global__ void __launch_bounds__(32) k_cpe_nnls(int64_t nprob, const double2* _
       if (++outer > 3 * ng) {
         status = 2;
         break;
-      }
-      if (p == cap && cap < ng) {
-        if (lane == 0) info[prob] = kNnlsRedo;
-        return;
       }
       if (!chol_append(S, N, ng, p, best, yv, lane)) {
         status = 3;
@@ -507,8 +478,8 @@ __global__ void __launch_bounds__(32) k_cpe_nnls(int64_t nprob, const double2* _
   }
 }
 
-__host__ __device__ constexpr size_t nnls_smem_bytes(int cap) {  // rows of the factor
-  return sizeof(double) * ((size_t)tri(cap) + 4 * kCpeMaxGrid) + sizeof(int) * 3 * kCpeMaxGrid;
+__host__ __device__ constexpr size_t nnls_smem_bytes(int ng) {
+  return sizeof(double) * ((size_t)tri(ng) + 4 * kCpeMaxGrid) + sizeof(int) * 3 * kCpeMaxGrid;
 }
 
 // Real-axis values and QP root, one warp per problem: the 401 scan points are split over
@@ -750,6 +721,8 @@ gw_status launch_continue(gw_ctx* c, int method, int64_t nprob, const double* si
     }
     c->cpe_b_bytes = need;
   }
+  const size_t smem = nnls_smem_bytes(c->cpe_ngrid);
+  cudaFuncSetAttribute(k_cpe_nnls, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   c->cpe_nprob = nprob;
   if ((size_t)nprob * sizeof(int) > c->cpe_iters_bytes) {
     if (c->d_cpe_iters) cudaFree(c->d_cpe_iters);
@@ -764,25 +737,10 @@ gw_status launch_continue(gw_ctx* c, int method, int64_t nprob, const double* si
   const double* seed = nullptr;
   if (c->cpe_seed_nprob == nprob) seed = c->d_cpe_seed;  // a seed set by gw_cpe_seed, consumed once
   c->cpe_seed_nprob = 0;
-  // A warp's time is a chain of latencies, so what counts is how many problems are resident: a factor of all
-  // 128 rows takes 72 KB, three per SM. When that leaves problems waiting, the first launch keeps 64 rows (ten per
-  // SM; passive sets have some tens of variables) and the few that outgrow them are done again, from the start and
-  // with the same values, by a second launch that skips the rest. Nk 27, Nb 32 (864 problems): 3.12 -> 2.13 ms.
-  const int ng = c->cpe_ngrid;
-  const size_t full = nnls_smem_bytes(ng), part = nnls_smem_bytes(kNnlsRows);
-  cudaFuncSetAttribute(k_cpe_nnls, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)full);
-  int sms = 0, res = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, k_cpe_nnls, 32, full) != cudaSuccess) res = 0;
-  const bool two = ng > kNnlsRows && nprob > (int64_t)res * sms;
-  gw_status s = GW_OK;
-  for (int redo = 0; redo <= two; ++redo) {
-    const bool all = !two || redo;
-    k_cpe_nnls<<<(unsigned)nprob, 32, all ? full : part, c->stream>>>(nprob, (const double2*)sig_iw, c->ncont, c->d_cpe_A,
-                                                                     c->d_cpe_N, ng, seed, c->d_cpe_b, info,
-                                                                     c->d_cpe_iters, all ? ng : kNnlsRows, redo);
-    if ((s = check_launch(c, "cpe_nnls")) != GW_OK) return s;
-  }
+  k_cpe_nnls<<<(unsigned)nprob, 32, smem, c->stream>>>(nprob, (const double2*)sig_iw, c->ncont, c->d_cpe_A, c->d_cpe_N,
+                                                     c->cpe_ngrid, seed, c->d_cpe_b, info, c->d_cpe_iters);
+  gw_status s = check_launch(c, "cpe_nnls");
+  if (s != GW_OK) return s;
   k_cpe_qp<<<(unsigned)((nprob + 3) / 4), 128, 0, c->stream>>>(nprob, c->d_cpe_b, c->d_cpe_x, c->cpe_ngrid,
                                                                  c->d_cpe_tab, eps,
                                                                  sigx, vxc, nreal, omega_real, (double2*)sig_real,
