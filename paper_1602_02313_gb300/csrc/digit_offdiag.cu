@@ -3,7 +3,7 @@
 //   GEMM 1   Z_jm(tau) = G_j(tau) W~(tau) a_jm            rows (k, j, m), columns I (Re, Im), K = J
 //   GEMM 2   Sigma_nm(k|tau) = pref sum_jI conj(a_jn^I) Z_jm^I(tau)   rows (tau, m) of a k, columns n, K = (j, I)
 // and Sigma^x as one more "tau" of GEMM 2 with Z_jm^I = occ_j v_I a_jm^I. Z is FP64 in between. k points and
-// tau go in groups whose Z and digits fit the workspace budget.
+// tau go in groups whose operands and Z fit 2 GiB.
 // Bound: the products' shared-memory operand rate (34 MMAs of 48 clocks per 16 K, digit_gemm.cuh) and, for Z, writing it,
 // its digits and reading both (44 bytes per element twice). Measured at Nk 8, Nb 32, NI 128, 16 tau: Sigma^c and Sigma^x
 // 29.5 -> 1.0 ms against the CUDA-core kernels of offdiag.cu (GEMM 1 0.61, GEMM 2 0.20, digits of Z 0.11). GEMM 2 has

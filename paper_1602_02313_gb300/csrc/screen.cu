@@ -275,17 +275,28 @@ __global__ void __launch_bounds__(256, AR::kBlocksPerSm) k_screen_inv(const doub
         for (int m = 0; m < 8; ++m)
 #pragma unroll
           for (int q = 0; q < 4; ++q) acc[m][q] = AR::azero();
-        for (int j = 0; j < GJ_B; ++j) {
-          S uq[4];
+        auto rank32 = [&](auto masked) {
+          for (int j = 0; j < GJ_B; ++j) {
+            S uq[4];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) uq[q] = U[j * (GJ_B + 1) + 4 * tc + q];
+            for (int q = 0; q < 4; ++q) uq[q] = U[j * (GJ_B + 1) + 4 * tc + q];
 #pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            if (!(rows >> m & 1)) continue;
-            const S l = L[(tr + 32 * m) * (GJ_B + 1) + j];
+            for (int m = 0; m < 8; ++m) {
+              if (decltype(masked)::value && !(rows >> m & 1)) continue;
+              const S l = L[(tr + 32 * m) * (GJ_B + 1) + j];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) AR::mac(acc[m][q], l, uq[q]);
+              for (int q = 0; q < 4; ++q) AR::mac(acc[m][q], l, uq[q]);
+            }
           }
+        };
+        if constexpr (kF32) {
+          // an FP32 product costs about what the test does (NI 256: 2.16 ms without it, 2.29 with it)
+          if (__popc(rows) > 4)
+            rank32(std::false_type{});
+          else
+            rank32(std::true_type{});
+        } else {
+          rank32(std::true_type{});
         }
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
