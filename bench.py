@@ -516,7 +516,7 @@ def run_offdiag(args):
 
 def run_gap_check(args):
     """The metric's accuracy claim on the benchmarked crystal (nk64_nb64, all 64 q): one G0W0 iteration
-    in FP64 (every step FP64) and in the mixed form (tensor-core P and Sigma^c, float-float or FP32
+    in FP64 (every step FP64) and in the mixed form (tensor-core P and Sigma^c, GW_F32X2 or FP32
     dielectric solve), the same continuation applied to both: CPE at ridges 1e-3, 1e-4, 1e-5 and Pade.
     Reports each chain's quasiparticle gap, the gap differences and the largest QP-energy difference
     (meV), the |Sigma| scale and the FP64 iteration time. A measurement run, not a bench line."""
@@ -644,11 +644,11 @@ def run_mlp(args):
 def run_c3(args):
     """The nk216_nb128 workload as a whole: all 216 q of the Nk = 216 (6x6x6), Nb = 128 (48
     occupied), NI = 512, Ntau = Nnu = Nw = 64, beta = 400 crystal, mixed precision (tensor-core P and
-    Sigma^c, float-float screening and bosonic transforms), one G0W0 iteration and args.c3_passes
+    Sigma^c, GW_F32X2 screening and bosonic transforms), one G0W0 iteration and args.c3_passes
     self-consistent passes (P, W~ and Sigma from the previous pass's dressed G), CPE continuation.
     Prints one JSON line per pass (time, gap, the change of G) and, first, per-quantity errors of
     this precision at sampled points: P of one q at two tau and Sigma^c of that q at sampled (k, tau)
-    (with a Hermitian stand-in for W~(tau)) against the FP64 oracle, and the float-float dielectric
+    (with a Hermitian stand-in for W~(tau)) against the FP64 oracle, and the GW_F32X2 dielectric
     solve of that q against the FP64 one on the GPU. A measurement run."""
     import torch
 
@@ -823,7 +823,7 @@ def main():
     ap.add_argument("--impl", default="gw", choices=["gw", "reference"])
     ap.add_argument("--prec", default="fp16x2", choices=["fp16x2", "fp64"])
     ap.add_argument("--screen", default="f32x2", choices=["f32x2", "f32"],
-                    help="arithmetic of the dielectric solve on the mixed chain: float-float (FP64-grade, the "
+                    help="arithmetic of the dielectric solve on the mixed chain: GW_F32X2 (FP64-grade, the "
                          "default) or plain FP32")
     ap.add_argument("--config", default="nk64_nb64")
     ap.add_argument("--omega", type=float, default=None,

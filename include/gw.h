@@ -48,7 +48,7 @@ typedef enum {
                      errors below an FP64 accumulation's; the rest native FP64); the parity path */
   GW_FP16X2 = 1,  /* tcgen05 tensor cores: fp16 hi/lo split operands, 3 products, FP32 TMEM accumulation */
                   /* (value 2 is not used) */
-  GW_F32X2 = 3,   /* float-float on the FP32 pipes: each value hi + lo in two FP32 (~44-bit significand) */
+  GW_F32X2 = 3,   /* FP64-grade: exact digit products on the tensor cores, float-float (hi + lo, ~44 bits) in the rest */
   GW_F32 = 4      /* plain FP32 on the CUDA cores (gw_screen only) */
 } gw_prec;
 
@@ -386,7 +386,7 @@ gw_status gw_kernel_timing(gw_ctx* ctx, int enable);
 
 /* Measured rates of the CUDA-core pipes on `device` (no context needed; runs two short
  * kernels of independent FMA chains): native FP64 and FP32 FMA throughput, TFLOP/s. A
- * float-float complex multiply-add (the mixed chain's screening and bosonic transforms) is 48
+ * float-float complex multiply-add (the mixed chain's exchange sum and pivot blocks) is 48
  * FP32-pipe operations, so fp32_tflops / 96 * 1e3 G/s is those kernels' ALU roofline.
  * Allocates 64 bytes. */
 gw_status gw_measure_alu(int device, double* fp64_tflops, double* fp32_tflops);

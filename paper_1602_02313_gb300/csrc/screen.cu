@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(256, AR::kBlocksPerSm) k_screen_inv(const doub
     // (A_iR <- -A_iR A_RR^-1 for the column block R, which starts from zero); the pass's
     // A_iR are taken into shared memory before its column block R is overwritten
     for (int r0 = 0; r0 < ni; r0 += GJ_RP) {
-      // bit m: rows r0 + 32 m .. + 31 exist and are not R. The others' products are left out: at NI = 64 that is
-      // seven of eight (1.50 -> 0.61 ms for 128 FP64 systems)
+      // bit m: rows r0 + 32 m .. + 31 exist and are not R. The others' products are left out (not in FP32): at
+      // NI = 64 that is seven of eight (1.50 -> 0.61 ms for 128 FP64 systems)
       unsigned rows = 0;
 #pragma unroll
       for (int m = 0; m < GJ_RP / GJ_B; ++m)
@@ -275,28 +275,18 @@ __global__ void __launch_bounds__(256, AR::kBlocksPerSm) k_screen_inv(const doub
         for (int m = 0; m < 8; ++m)
 #pragma unroll
           for (int q = 0; q < 4; ++q) acc[m][q] = AR::azero();
-        auto rank32 = [&](auto masked) {
-          for (int j = 0; j < GJ_B; ++j) {
-            S uq[4];
+        for (int j = 0; j < GJ_B; ++j) {
+          S uq[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) uq[q] = U[j * (GJ_B + 1) + 4 * tc + q];
+          for (int q = 0; q < 4; ++q) uq[q] = U[j * (GJ_B + 1) + 4 * tc + q];
 #pragma unroll
-            for (int m = 0; m < 8; ++m) {
-              if (decltype(masked)::value && !(rows >> m & 1)) continue;
-              const S l = L[(tr + 32 * m) * (GJ_B + 1) + j];
+          for (int m = 0; m < 8; ++m) {
+            // (an FP32 product costs about what the test does: NI 256 2.16 ms without it, 2.29 with it)
+            if (!kF32 && !(rows >> m & 1)) continue;
+            const S l = L[(tr + 32 * m) * (GJ_B + 1) + j];
 #pragma unroll
-              for (int q = 0; q < 4; ++q) AR::mac(acc[m][q], l, uq[q]);
-            }
+            for (int q = 0; q < 4; ++q) AR::mac(acc[m][q], l, uq[q]);
           }
-        };
-        if constexpr (kF32) {
-          // an FP32 product costs about what the test does (NI 256: 2.16 ms without it, 2.29 with it)
-          if (__popc(rows) > 4)
-            rank32(std::false_type{});
-          else
-            rank32(std::true_type{});
-        } else {
-          rank32(std::true_type{});
         }
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
