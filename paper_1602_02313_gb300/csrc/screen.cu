@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256, AR::kBlocksPerSm) k_screen_inv(const doub
   using Acc = typename AR::Acc;
   extern __shared__ __align__(16) unsigned char gsm_raw[];
   S* Pinv = reinterpret_cast<S*>(gsm_raw);  // [32][33]
-  S* L = Pinv + GJ_B * (GJ_B + 1);           // [GJ_RP][33]: A[i][R] of one row pass (not the rows of R)
+  S* L = Pinv + GJ_B * (GJ_B + 1);           // [GJ_RP][33]: A[i][R] of one row pass (rows of R zeroed or left out)
   S* U = L + (size_t)GJ_RP * (GJ_B + 1);     // [32][33]
   __shared__ int bad;
   __shared__ S fcol[GJ_B], rowj[GJ_B];
@@ -252,15 +252,19 @@ __global__ void __launch_bounds__(256, AR::kBlocksPerSm) k_screen_inv(const doub
     // (A_iR <- -A_iR A_RR^-1 for the column block R, which starts from zero); the pass's
     // A_iR are taken into shared memory before its column block R is overwritten
     for (int r0 = 0; r0 < ni; r0 += GJ_RP) {
-      // bit m: rows r0 + 32 m .. + 31 exist and are not R. The others' products are left out (not in FP32): at
-      // NI = 64 that is seven of eight (1.50 -> 0.61 ms for 128 FP64 systems)
+      // bit m: rows r0 + 32 m .. + 31 exist and are not R. The others' products are left out: at NI = 64
+      // seven of eight (1.50 -> 0.61 ms for 128 FP64 systems). Not in FP32, where a product costs about what the
+      // test does (NI 256: 2.16 ms without it, 2.29 with it).
       unsigned rows = 0;
 #pragma unroll
       for (int m = 0; m < GJ_RP / GJ_B; ++m)
         if (r0 + GJ_B * m < ni && r0 + GJ_B * m != k0) rows |= 1u << m;
       for (int e = t; e < GJ_RP * GJ_B; e += blockDim.x) {
-        const int r = e / GJ_B, c = e % GJ_B;
-        if (rows >> (r / GJ_B) & 1) L[r * (GJ_B + 1) + c] = A[(size_t)(r0 + r) * ni + k0 + c];
+        const int r = e / GJ_B, c = e % GJ_B, gr = r0 + r;
+        if constexpr (kF32)
+          L[r * (GJ_B + 1) + c] = (gr >= ni || (gr >= k0 && gr < k0 + GJ_B)) ? AR::zero() : A[(size_t)gr * ni + k0 + c];
+        else if (rows >> (r / GJ_B) & 1)
+          L[r * (GJ_B + 1) + c] = A[(size_t)gr * ni + k0 + c];
       }
       for (int c0 = 0; c0 < ni; c0 += GJ_B) {
         const bool isR = c0 == k0;
@@ -281,7 +285,6 @@ __global__ void __launch_bounds__(256, AR::kBlocksPerSm) k_screen_inv(const doub
           for (int q = 0; q < 4; ++q) uq[q] = U[j * (GJ_B + 1) + 4 * tc + q];
 #pragma unroll
           for (int m = 0; m < 8; ++m) {
-            // (an FP32 product costs about what the test does: NI 256 2.16 ms without it, 2.29 with it)
             if (!kF32 && !(rows >> m & 1)) continue;
             const S l = L[(tr + 32 * m) * (GJ_B + 1) + j];
 #pragma unroll
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(256, AR::kBlocksPerSm) k_screen_inv(const doub
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
           const int r = r0 + tr + 32 * m;
-          if (!(rows >> m & 1)) continue;
+          if (kF32 ? r >= ni || (r >= k0 && r < k0 + GJ_B) : !(rows >> m & 1)) continue;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             S* a = &A[(size_t)r * ni + c0 + 4 * tc + q];
