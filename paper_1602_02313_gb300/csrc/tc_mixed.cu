@@ -36,6 +36,7 @@
 
 #include "cvt.cuh"
 #include "gw_internal.h"
+#include "pol_plan.h"
 #include "tc_common.cuh"
 
 namespace gwi {
@@ -162,11 +163,14 @@ struct PolJob {
 };
 
 // Barrier phases of a block that runs several work units one after another, kept by every role for
-// itself: bit s of `ph` is the phase of stage s's next use; the MMA warp commits `done` once per unit.
+// itself: bit s of `ph` is the phase of stage s's next use; the MMA warp commits `done` once per unit that has
+// chunks. The next commit of `done` waits for operands that the epilogue's warps build after their wait for this
+// one; a unit without chunks has no such wait, so a commit of its own could move the barrier a second phase on
+// under warps still waiting for the first.
 struct PolPhase {
   uint32_t ph = 0;
   int s = 0;      // next stage (0 at the start of a unit that may change the number of stages)
-  int units = 0;  // units already run (commits of `done`)
+  int units = 0;  // commits of `done` so far
   uint32_t used = 0, uph = 0;  // copy thread: stages ever filled, and the phase of each one's last copy
 };
 
@@ -193,7 +197,7 @@ __device__ __forceinline__ void pol_unit(const PolJob& J, int u, PolSmem& S, uns
   const int xb = sd.x, c0 = sd.y, N = sd.z;
   const int nib = (J.ni + 127) / 128;
   const int total = J.nk * cpk;
-  const int L = (total + J.nseg - 1) / J.nseg;
+  const int L = pol_seg_len(total, J.nseg);
   const int g0 = seg * L, g1 = min(total, g0 + L);
   const int nchunk = max(0, g1 - g0);
   // stages of hps halves; in a stage X of its halves (each [tau][hi, lo]), then Y of its halves ([hi, lo])
@@ -373,7 +377,7 @@ __device__ __forceinline__ void pol_unit(const PolJob& J, int u, PolSmem& S, uns
         pol_next(ph, nst);
       }
     }
-    if (lead) mma_commit(&S.done);
+    if (lead && nchunk) mma_commit(&S.done);
     __syncwarp();
   } else {
     // ------------------------------------------------------------ copies of Y, by one lane
@@ -431,7 +435,7 @@ __device__ __forceinline__ void pol_unit(const PolJob& J, int u, PolSmem& S, uns
     }
     tc_fence_before();
   }
-  ph.units += 1;
+  ph.units += nchunk > 0;
 }
 
 __device__ __forceinline__ void pol_block_init(PolSmem& S, int tid, int warp) {
@@ -1065,8 +1069,7 @@ static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
   const int sms = num_sms(c);
   const int base_units = nstrips * c->ntau;
   const int seg_chunks = std::max(1, std::min(c->pol_seg_chunks, kPolChunksPerSeg));
-  int nseg = std::max(1, (total + seg_chunks - 1) / seg_chunks);
-  while (base_units * nseg < 2 * sms && (total + nseg) / (nseg + 1) >= 4) ++nseg;
+  const int nseg = pol_segments(total, base_units, seg_chunks, sms);
   // the partials of at most pol_part_bytes are held at once: segments run in passes, each
   // reduced into P (the first pass writes, later ones add)
   const size_t seg_bytes = (size_t)base_units * (eform ? 1 : 2) * P_TILE * sizeof(float);  // E form: units of two tau
