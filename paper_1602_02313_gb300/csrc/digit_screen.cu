@@ -19,6 +19,7 @@
 
 #include "arith.cuh"
 #include "digit_gemm.cuh"
+#include "gj_block.cuh"
 
 namespace gwi {
 
@@ -69,10 +70,15 @@ __global__ void k_gj_out(const double2* __restrict__ A, const double* __restrict
   W[(sys0 + s) * nn + e] = make_double2(q * (x.x - (I == J ? 1.0 : 0.0)), q * x.y);
 }
 
+struct BlockSync {
+  __device__ __forceinline__ void block() const { __syncthreads(); }
+  __device__ __forceinline__ void warp() const { __syncwarp(); }
+};
+
 // One system per block: P = A_RR^-1 in float-float, written in FP64 (to P and, when R is the whole matrix,
 // to A) and as digits: row 2 r = [Re P_r | -Im P_r], 2 r + 1 = [Im P_r | Re P_r]. In-place Gauss-Jordan by
-// two 32-wide blocks H: H's 32 x 32 inverse by elimination with 2 x 2 elements per thread in registers (a
-// step moves only its row and column through shared memory), then three 32^3 products for the other half.
+// two 32-wide blocks H: H's 32 x 32 inverse by elimination with 2 x 2 elements per thread in registers
+// (gj_block.cuh; a step moves only its row and column through shared memory), then three 32^3 products for the other half.
 // Summing 32 products before one subtraction keeps the error below that of 64 elimination steps (1.2e-14
 // against 0.8e-14 for random matrices), and the steps are short: ALU-bound (64^3 complex multiply-adds of
 // 48 operations) with two or three blocks per SM.
@@ -96,41 +102,11 @@ __global__ void __launch_bounds__(256, 3) k_gj_pivot(GjJob J, int sys0, int* __r
     for (int a = 0; a < 2; ++a)
 #pragma unroll
       for (int b = 0; b < 2; ++b) x[a][b] = H[(ty + 16 * a) * GJ_LD + tx + 16 * b];
-    // row j <- row j / p (entry j -> 1 / p); other rows r: a_rc -= a_rj a_jc / p, a_rj <- -a_rj / p
-#pragma unroll
-    for (int jb = 0; jb < 2; ++jb)
-      for (int jj = 0; jj < 16; ++jj) {
-        const int j = 16 * jb + jj;
-        if (tx == jj) {
-          fcol[ty] = Ff32::neg(x[0][jb]);
-          fcol[ty + 16] = Ff32::neg(x[1][jb]);
-        }
-        if (ty == jj) {
-          prow[tx] = x[jb][0];
-          prow[tx + 16] = x[jb][1];
-        }
-        __syncthreads();
-        const S p = prow[j];
-        if (Ff32::is_zero(p)) {
-          if (t == 0) info[sys0 + s] = J.k0 + h0 + j + 1;
-          return;
-        }
-        if (t < 32) {
-          const S ip = Ff32::inv(p);
-          rowj[t] = t == j ? ip : Ff32::fma2(Ff32::zero(), prow[t], ip);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            const S g = rowj[tx + 16 * b];
-            S v = x[a][b];
-            if (b == jb && tx == jj) v = Ff32::zero();
-            v = Ff32::fma2(v, fcol[ty + 16 * a], g);
-            x[a][b] = a == jb && ty == jj ? g : v;
-          }
-      }
+    const int zero = gj_invert32<Ff32>(x, fcol, prow, rowj, t, BlockSync());
+    if (zero >= 0) {
+      if (t == 0) info[sys0 + s] = J.k0 + h0 + zero + 1;
+      return;
+    }
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
