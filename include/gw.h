@@ -393,7 +393,9 @@ gw_status gw_measure_alu(int device, double* fp64_tflops, double* fp32_tflops);
 
 /* Moves the context to another cudaStream_t (same device) for the calls that follow; work
  * already queued stays on the old stream (the caller orders the two). Lets one context serve as
- * a branch of a multi-stream CUDA graph. NULL = the legacy default stream. */
+ * a branch of a multi-stream CUDA graph. NULL = the legacy default stream.
+ * Workspaces grow on use. From the first call that was captured on the context, an outgrown one is kept until
+ * gw_destroy, so that graphs captured earlier stay valid whatever is called later. */
 gw_status gw_set_stream(gw_ctx* ctx, void* stream);
 
 /* Knobs of the tensor-core contractions.

@@ -711,29 +711,12 @@ gw_status launch_continue(gw_ctx* c, int method, int64_t nprob, const double* si
     return check_launch(c, "pade");
   }
   const size_t need = (size_t)nprob * c->cpe_ngrid * sizeof(double);
-  if (need > c->cpe_b_bytes) {
-    if (c->d_cpe_b) cudaFree(c->d_cpe_b);
-    c->d_cpe_b = nullptr;
-    c->cpe_b_bytes = 0;
-    if (cudaMalloc((void**)&c->d_cpe_b, need) != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(c, GW_ENOMEM, "cpe workspace");
-    }
-    c->cpe_b_bytes = need;
-  }
+  if (!grow_ws(c, (void**)&c->d_cpe_b, &c->cpe_b_bytes, need)) return set_err(c, GW_ENOMEM, "cpe workspace");
   const size_t smem = nnls_smem_bytes(c->cpe_ngrid);
   cudaFuncSetAttribute(k_cpe_nnls, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   c->cpe_nprob = nprob;
-  if ((size_t)nprob * sizeof(int) > c->cpe_iters_bytes) {
-    if (c->d_cpe_iters) cudaFree(c->d_cpe_iters);
-    c->d_cpe_iters = nullptr;
-    c->cpe_iters_bytes = 0;
-    if (cudaMalloc((void**)&c->d_cpe_iters, nprob * sizeof(int)) != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(c, GW_ENOMEM, "cpe iteration counts");
-    }
-    c->cpe_iters_bytes = nprob * sizeof(int);
-  }
+  if (!grow_ws(c, (void**)&c->d_cpe_iters, &c->cpe_iters_bytes, nprob * sizeof(int)))
+    return set_err(c, GW_ENOMEM, "cpe iteration counts");
   const double* seed = nullptr;
   if (c->cpe_seed_nprob == nprob) seed = c->d_cpe_seed;  // a seed set by gw_cpe_seed, consumed once
   c->cpe_seed_nprob = 0;
@@ -864,16 +847,7 @@ extern "C" gw_status gw_cpe_fit_matrix(gw_ctx* c, int nfit, float* A) {
 extern "C" gw_status gw_cpe_seed(gw_ctx* c, int64_t nprob, const float* bhat, const double* scale) {
   if (!c || nprob <= 0 || !bhat || !scale || c->cpe_ngrid == 0) return GW_EINVAL;
   const size_t need = (size_t)nprob * c->cpe_ngrid * sizeof(double);
-  if (need > c->cpe_seed_bytes) {
-    if (c->d_cpe_seed) cudaFree(c->d_cpe_seed);
-    c->d_cpe_seed = nullptr;
-    c->cpe_seed_bytes = 0;
-    if (cudaMalloc((void**)&c->d_cpe_seed, need) != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(c, GW_ENOMEM, "cpe seed");
-    }
-    c->cpe_seed_bytes = need;
-  }
+  if (!grow_ws(c, (void**)&c->d_cpe_seed, &c->cpe_seed_bytes, need)) return set_err(c, GW_ENOMEM, "cpe seed");
   const int64_t n = nprob * c->cpe_ngrid;
   k_cpe_seed<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, c->cpe_ngrid, bhat, scale, c->d_cpe_seed);
   c->cpe_seed_nprob = nprob;

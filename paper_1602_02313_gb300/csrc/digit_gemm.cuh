@@ -354,26 +354,12 @@ __global__ void __launch_bounds__(X_THREADS, 1)
 }
 
 
-// Host side: the context's digit workspaces, one for each use (a call captured into a graph keeps its
-// workspace when another use grows), grown on use. False (nothing launched, no error set) when it cannot be
-// had: no memory, or a capture in progress, where nothing may be allocated; the callers then run kernels
-// that need none.
+// Host side: the context's digit workspaces, one for each use, grown on use (grow_ws: a captured call keeps
+// the one it was captured with). False (nothing launched, no error set) when it cannot be had: no memory, or a
+// capture in progress, where nothing may be allocated; the callers then run kernels that need none.
 inline bool x_workspace(gw_ctx* c, int use, size_t need) {
-  if (need <= c->x_ws_bytes[use]) return true;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
-  if (c->x_ws[use]) cudaFree(c->x_ws[use]);
-  c->x_ws[use] = nullptr;
-  c->x_ws_bytes[use] = 0;
-  if (cudaMalloc(&c->x_ws[use], need) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  c->x_ws_bytes[use] = need;
-  return true;
+  if (need > c->x_ws_bytes[use] && capturing(c)) return false;
+  return grow_ws(c, &c->x_ws[use], &c->x_ws_bytes[use], need);
 }
 enum { XW_POL = 0, XW_SIGMA = 1, XW_BOSE = 2, XW_SCREEN = 3, XW_OFFDIAG = 4 };
 

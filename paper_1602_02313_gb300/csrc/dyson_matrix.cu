@@ -412,16 +412,7 @@ extern "C" gw_status gw_dyson_matrix(gw_ctx* c, const double* eps, const double*
   const size_t b_hat = 2 * el * nw * sizeof(double2);
   const size_t b_g0 = (size_t)nk * nbp * (nt + 1) * sizeof(double);
   const size_t need = b_siw + b_eig + b_aug + b_hat + b_g0 + 1024;
-  if (need > c->dm_bytes) {
-    if (c->d_dm) cudaFree(c->d_dm);
-    c->d_dm = nullptr;
-    c->dm_bytes = 0;
-    if (cudaMalloc(&c->d_dm, need) != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(c, GW_ENOMEM, "gw_dyson_matrix: workspace");
-    }
-    c->dm_bytes = need;
-  }
+  if (!grow_ws(c, &c->d_dm, &c->dm_bytes, need)) return set_err(c, GW_ENOMEM, "gw_dyson_matrix: workspace");
   char* w = (char*)c->d_dm;
   double2* Siw = Sc_tau ? (double2*)w : nullptr;
   w += b_siw;

@@ -519,6 +519,36 @@ __global__ void k_sigx_occ(const double* __restrict__ vm, const int* __restrict_
   Sx[e] += pref * s;
 }
 
+bool capturing(gw_ctx* c) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    cs = cudaStreamCaptureStatusActive;
+  }
+  if (cs != cudaStreamCaptureStatusNone) c->captured = true;
+  return cs != cudaStreamCaptureStatusNone;
+}
+
+bool grow_ws(gw_ctx* c, void** p, size_t* have, size_t need) {
+  capturing(c);
+  if (need <= *have) return true;
+  if (*p) {
+    if (c->captured)
+      c->retired.push_back(*p);
+    else
+      cudaFree(*p);
+  }
+  *p = nullptr;
+  *have = 0;
+  if (cudaMalloc(p, need) != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+    return false;
+  }
+  *have = need;
+  return true;
+}
+
 gw_status launch_sigx(gw_ctx* c, int iq, const double* occ, double* Sx, bool ff) {
   const int np = c->nb * c->nb;
   const size_t need = (size_t)c->nk * np * sizeof(double);
@@ -721,6 +751,7 @@ gw_status gw_destroy(gw_ctx* c) {
   if (c->d_dm) cudaFree(c->d_dm);
   for (void* p : c->x_ws)
     if (p) cudaFree(p);
+  for (void* p : c->retired) cudaFree(p);
   if (c->d_bdig) cudaFree(c->d_bdig);
   double* bufs[] = {c->d_sqrtv, c->d_v,       c->d_M_own, c->d_Bfwd,  c->d_Ffwd,  c->d_Fcont, c->d_Bbwd,
                     c->d_Fbwd,  c->d_Fbwd_beta, c->d_aug,   c->d_cpe_x, c->d_cpe_A, c->d_cpe_N, c->d_cpe_tab, c->d_cpe_b,
@@ -865,16 +896,7 @@ gw_status gw_tau_to_freq(gw_ctx* c, gw_stat stat, gw_dir dir, int64_t batch, con
 gw_status gw_screen(gw_ctx* c, int iq0, int nqb, const double* P, gw_prec prec, double* W, int* info) {
   if (!c || !P || !W || !info || iq0 < 0 || nqb < 1 || iq0 + nqb > c->nq) return GW_EINVAL;
   const size_t need = (size_t)nqb * c->nnu * c->ni * 2 * c->ni * sizeof(double2);
-  if (need > c->aug_bytes) {
-    if (c->d_aug) cudaFree(c->d_aug);
-    c->d_aug = nullptr;
-    c->aug_bytes = 0;
-    if (cudaMalloc((void**)&c->d_aug, need) != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(c, GW_ENOMEM, "gw_screen: workspace");
-    }
-    c->aug_bytes = need;
-  }
+  if (!grow_ws(c, (void**)&c->d_aug, &c->aug_bytes, need)) return set_err(c, GW_ENOMEM, "gw_screen: workspace");
   return launch_screen(c, iq0, nqb, (int)prec, P, W, info, c->d_aug);
 }
 

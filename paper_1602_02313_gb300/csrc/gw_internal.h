@@ -115,6 +115,8 @@ struct gw_ctx {
   void* x_ws[5] = {};           // digit products on the tensor cores: operand digits, partial sums
   size_t x_ws_bytes[5] = {};
   void* d_bdig = nullptr;       // digits of the bosonic maps (digit_bose.cu)
+  bool captured = false;        // a call was captured into a graph, which keeps the workspaces it saw
+  std::vector<void*> retired;   // workspaces outgrown since: freed with the context
   // tensor-core path
   gwi::MixedWork mw;
   int* d_err = nullptr;                     // error word of the bounded device waits (read by gw_sync)
@@ -140,6 +142,13 @@ gw_status check_launch(gw_ctx* c, const char* what);
 void kt_begin(gw_ctx* c, const char* name);
 void kt_end(gw_ctx* c);
 gw_status set_err(gw_ctx* c, gw_status s, const std::string& msg);
+// whether the context's stream is being captured (or may be); remembered in c->captured
+bool capturing(gw_ctx* c);
+// Makes the workspace *p of *have bytes hold at least `need`; false when the memory cannot be had (*p is then
+// null). Every call that uses a workspace which may grow later comes through here, also when it is large
+// enough: from the first captured one on, an outgrown buffer is kept until gw_destroy instead of freed, since
+// a graph replays with the addresses it was captured with.
+bool grow_ws(gw_ctx* c, void** p, size_t* have, size_t need);
 
 gw_status launch_gen_m(gw_ctx* c, double* M);
 // device address of M[iq] ([nk][ni][nb][nb] cplx); with per-q generation, (re)generates the

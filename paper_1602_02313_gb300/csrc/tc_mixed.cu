@@ -1005,15 +1005,7 @@ __global__ void k_sig_reduce(const double* __restrict__ D, const double* __restr
 
 // ------------------------------------------------------------------ workspace helpers
 gw_status ensure(gw_ctx* c, void** p, size_t* have, size_t need, const char* what) {
-  if (need <= *have) return GW_OK;
-  if (*p) cudaFree(*p);
-  *p = nullptr;
-  *have = 0;
-  if (cudaMalloc(p, need) != cudaSuccess) {
-    cudaGetLastError();
-    return set_err(c, GW_ENOMEM, std::string("tensor-core workspace: ") + what);
-  }
-  *have = need;
+  if (!grow_ws(c, p, have, need)) return set_err(c, GW_ENOMEM, std::string("tensor-core workspace: ") + what);
   return GW_OK;
 }
 
