@@ -44,8 +44,14 @@ typedef enum {
 
 /* Arithmetic of the P and Sigma^c contractions. */
 typedef enum {
-  GW_FP64 = 0,    /* FP64 (P, Sigma^c: exact fp16 digit products on the tensor cores, summed in integers, with
-                     errors below an FP64 accumulation's; the rest native FP64); the parity path */
+  GW_FP64 = 0,    /* FP64; the parity path. P, Sigma^c and the off-diagonal self-energy are sums x y over rows x
+                     and y of two operands, formed by exact fp16 digit products on the tensor cores and summed in
+                     integers (native FP64 with GW_TUNE_FP64_FORM 1, or where their workspace cannot be had).
+                     Every row is cut at 2^-56 of its own largest entry, so the error of a sum of n terms is at
+                     most n 2^-50 max|x| max|y| (2^-56 sqrt(n) max|x| max|y| in the root mean square): below that
+                     of an FP64 accumulation for rows of one scale, but relative to the rows' largest entries, not
+                     to each term. Where large entries of x meet only tiny ones of y and the other way round, the
+                     small sum that remains has fewer correct digits than FP64 gives it. The rest is native FP64. */
   GW_FP16X2 = 1,  /* tcgen05 tensor cores: fp16 hi/lo split operands, 3 products, FP32 TMEM accumulation */
                   /* (value 2 is not used) */
   GW_F32X2 = 3,   /* FP64-grade: exact digit products on the tensor cores, float-float (hi + lo, ~44 bits) in the rest */
@@ -411,14 +417,19 @@ gw_status gw_set_stream(gw_ctx* ctx, void* stream);
  *      nothing arrives on, so the wait runs out after the wait budget (the GPU stays usable);
  *  GW_TUNE_POL_FORM: how the tensor-core polarization covers the Hermitian P(tau): 0 = by ni (the
  *      default: the real matrix E = Re P + Im P for ni <= 256, Re P and Im P over the Hermitian
- *      half above), 1 = always E, 2 = always Re P and Im P. Both give P within the same bound.
- * Out-of-range values return GW_EINVAL. Results stay within the tensor-core error bound. */
+ *      half above), 1 = always E, 2 = always Re P and Im P. Both give P within the same bound;
+ *  GW_TUNE_FP64_FORM: how gw_polarization and gw_selfenergy with GW_FP64, and gw_selfenergy_offdiag, sum:
+ *      0 = digit products on the tensor cores (the default; errors relative to the largest entries of the
+ *      rows, see GW_FP64), 1 = native FP64 on the CUDA cores (errors relative to each term; 15 to 57 times
+ *      slower, no workspace).
+ * Out-of-range values return GW_EINVAL. Results stay within the error bound of their arithmetic. */
 typedef enum {
   GW_TUNE_POL_SEG_CHUNKS = 0,
   GW_TUNE_POL_PART_MB = 1,
   GW_TUNE_WAIT_CYCLES = 2,
   GW_TUNE_FAULT_STALL = 3,
-  GW_TUNE_POL_FORM = 4
+  GW_TUNE_POL_FORM = 4,
+  GW_TUNE_FP64_FORM = 5
 } gw_tune;
 gw_status gw_set_tuning(gw_ctx* ctx, gw_tune key, int64_t value);
 gw_status gw_kernel_time(gw_ctx* ctx, const char* kernel, double* total_ms, int64_t* launches);

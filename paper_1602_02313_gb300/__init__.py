@@ -25,6 +25,7 @@ GW_BOSE, GW_FERMI = 0, 1
 GW_TAU_TO_IW, GW_IW_TO_TAU, GW_TAU_TO_IW_CONT = 0, 1, 2
 GW_PADE, GW_CPE = 0, 1
 GW_TUNE_POL_SEG_CHUNKS, GW_TUNE_POL_PART_MB, GW_TUNE_WAIT_CYCLES, GW_TUNE_FAULT_STALL, GW_TUNE_POL_FORM = 0, 1, 2, 3, 4
+GW_TUNE_FP64_FORM = 5
 PREC = {"fp64": GW_FP64, "fp16x2": GW_FP16X2}
 
 _STATUS = {0: "GW_OK", -1: "GW_EINVAL", -2: "GW_ENOMEM", -3: "GW_ECUDA", -4: "GW_ESINGULAR",

@@ -1,6 +1,7 @@
 // FP64 (CUDA-core) forms of the two product-basis contractions, without any workspace: they run where
-// the tensor-core form (exact_tc.cu, 15 to 57 times faster) cannot have its digit workspace: no memory
-// left, or a first call under stream capture.
+// the tensor-core form (exact_tc.cu, 15 to 57 times faster) cannot have its digit workspace (no memory
+// left, or a first call under stream capture), and with GW_TUNE_FP64_FORM 1: their error is relative to
+// each term of a sum, the digit products' to the largest entries of its two rows.
 //
 // polarization, Eq. (irpol):  P_II'(q|tau) = 1/(Omega Nk) sum_k sum_ab M^I_ab Q_ab(tau) conj(M^I'_ab)
 //   Q_ab(tau) = G_b(k|tau) G_a(k-q|-tau) = -G_b(k|tau) G_a(k-q|beta - tau)   (Sec. II)

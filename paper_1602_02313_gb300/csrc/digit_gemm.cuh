@@ -9,9 +9,12 @@
 // tensor memory per level, over blocks of 192 k: |L_s| <= (s + 1) 192 2^14 < 2^24 for s <= 4, so the
 // FP32 sums are exact there (at s = 5, 6 an extreme coherent row could round, by 2^-54 of the sum of
 // |a b|). The blocks' levels are added up in 64-bit integers and become one double per element at
-// the end. What is lost is the rounding of each operand to 2^-56 of its row's largest value and the
-// levels above 6: smaller than the rounding errors an FP64 accumulation of the same sum makes (the
-// measured errors of P and Sigma^c against exact sums are below the CUDA-core kernels' over all tested sizes).
+// the end. What is lost is the rounding of each operand to 2^-56 of its row's scale 2^e (2^(e-1) <= max|x| < 2^e)
+// and the levels above 6: per term at most (2 + 6.03) 2^-56 2^(ea + eb), below 2^-50 max|a| max|b|; about 2^-56
+// 2^(ea + eb) in the root mean square. That is below the rounding errors of an FP64 accumulation for rows
+// whose entries are of one scale (measured errors of P and Sigma^c against exact sums on such data are below the
+// CUDA-core kernels'), but it is relative to the rows' largest entries: a = [1, 2^-60], b = [2^-60, 1] gives 0, where
+// FP64 gives 2^-59. GW_TUNE_FP64_FORM 1 takes the CUDA-core kernels, whose error is relative to each term.
 // Rows that hold an infinity or a nan give nan.
 //
 // Short sums leave FP64 fewer roundings to make: of the digits' loss most is the first level left out (six products,

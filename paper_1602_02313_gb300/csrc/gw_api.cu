@@ -819,6 +819,10 @@ gw_status gw_set_tuning(gw_ctx* c, gw_tune key, int64_t value) {
       if (value < 0 || value > 2) return set_err(c, GW_EINVAL, "gw_set_tuning: polarization form is 0, 1 or 2");
       c->pol_form = (int)value;
       return GW_OK;
+    case GW_TUNE_FP64_FORM:
+      if (value != 0 && value != 1) return set_err(c, GW_EINVAL, "gw_set_tuning: FP64 form is 0 or 1");
+      c->fp64_form = (int)value;
+      return GW_OK;
   }
   return set_err(c, GW_EINVAL, "gw_set_tuning: unknown key");
 }
@@ -857,7 +861,7 @@ gw_status gw_green_tau(gw_ctx* c, const double* eps, const double* sigx, const d
 gw_status gw_polarization(gw_ctx* c, int iq, const double* G, gw_prec prec, double* P) {
   if (!c || !G || !P || iq < 0 || iq >= c->nq) return GW_EINVAL;
   if (prec == GW_FP64) {
-    const gw_status st = launch_pol_exact(c, iq, G, P);
+    const gw_status st = c->fp64_form ? GW_EUNSUPPORTED : launch_pol_exact(c, iq, G, P);
     return st == GW_EUNSUPPORTED ? launch_pol_fp64(c, iq, G, P) : st;
   }
   if (prec == GW_FP16X2) return launch_pol_mixed(c, iq, G, (int)prec, P);
@@ -905,7 +909,7 @@ gw_status gw_selfenergy(gw_ctx* c, int iq, const double* G, const double* occ, c
   if (!c || !G || !W || !S || iq < 0 || iq >= c->nq || (Sx && !occ)) return GW_EINVAL;
   gw_status st;
   if (prec == GW_FP64) {
-    st = launch_sigma_exact(c, iq, G, W, S);
+    st = c->fp64_form ? GW_EUNSUPPORTED : launch_sigma_exact(c, iq, G, W, S);
     if (st == GW_EUNSUPPORTED) st = launch_sigma_fp64(c, iq, G, W, S);
   } else if (prec == GW_FP16X2)
     st = launch_sigma_mixed(c, iq, G, W, (int)prec, S);

@@ -122,6 +122,7 @@ struct gw_ctx {
   int* d_err = nullptr;                     // error word of the bounded device waits (read by gw_sync)
   long long wait_cycles = 4000000000ll;     // clock cycles a tensor-core pipeline wait may take (~2 s)
   int fault_stall = 0;                      // test fault injection: MMA issuers wait on a barrier nothing sets
+  int fp64_form = 0;                        // GW_FP64 contractions: 0 digit products, 1 CUDA cores (GW_TUNE_FP64_FORM)
   int pol_form = 0;                         // polarization cover: 0 by ni, 1 E = Re P + Im P, 2 Re P and Im P
   int pol_seg_chunks = 32;                  // K chunks per FP32 accumulation segment of P (<= 32)
   size_t pol_part_bytes = 8ull << 30;       // FP32 partial strips of P held at once

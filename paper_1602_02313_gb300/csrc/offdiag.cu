@@ -3,8 +3,8 @@
 //   Sigma^c_nm(k|tau) += -1/(Omega N_k) sum_j G_j(k - q|tau) sum_IJ conj(M^I_jn) W~_IJ(tau) M^J_jm
 //   Sigma^x_nm(k)     += -1/(Omega N_k) sum_j occ_j(k - q) sum_I v_I conj(M^I_jn) M^I_jm
 // By digit products on the tensor cores (digit_offdiag.cu: 29.5 -> 1.0 ms at Nk 8, Nb 32, NI 128,
-// 16 tau); without their workspace (no memory, a first call under capture) in FP64 on the CUDA cores
-// here. Sigma^c: one block per (k, tau); for each j and each chunk of ci rows I of W~(tau), the block
+// 16 tau); without their workspace (no memory, a first call under capture) or with GW_TUNE_FP64_FORM 1
+// in FP64 on the CUDA cores here. Sigma^c: one block per (k, tau); for each j and each chunk of ci rows I of W~(tau), the block
 // forms Z = W~(tau)[I chunk, :] a_j (ci x Nb, a_j = M[k][:, j, :]) in shared memory and adds
 // G_j a_j[I chunk]^+ Z to the Nb x Nb accumulator, also in shared memory, so any NI fits. Sigma^x:
 // one block per k.
@@ -103,7 +103,8 @@ extern "C" gw_status gw_selfenergy_offdiag(gw_ctx* c, int iq, const double* G_ta
   const size_t budget = 200 * 1024, acc_b = (size_t)nb * nb * sizeof(double2), row_b = (size_t)nb * sizeof(double2);
   if (acc_b + 8 * row_b > budget)
     return set_err(c, GW_EINVAL, "gw_selfenergy_offdiag: the nb x nb accumulator and 8 rows of W~ a_j need 16 nb^2 + 128 nb bytes <= 200 KiB (nb <= 109)");
-  const gw_status digits = launch_offdiag_digits(c, iq, G_tau, occ, W_tau, S_tau, Sx);
+  const gw_status digits =
+      c->fp64_form ? GW_EUNSUPPORTED : launch_offdiag_digits(c, iq, G_tau, occ, W_tau, S_tau, Sx);
   if (digits != GW_EUNSUPPORTED) return digits;
   int ci = (int)std::min<size_t>((size_t)ni, (budget - acc_b) / row_b);
   if (ci < ni) ci &= ~7;
