@@ -41,6 +41,8 @@ struct MixedWork {
   size_t dacc_bytes = 0;
   bool strips_ready = false;
   int strips_form = -1;       // the form the uploaded strips were built for
+  int pass_cap = 0;           // memory was short: at most this many K segments of P per pass (0: no limit)
+  bool no_xf = false;         // memory was short for the E form of P at one segment per pass
 };
 
 }  // namespace gwi

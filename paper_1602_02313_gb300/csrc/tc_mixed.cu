@@ -1031,14 +1031,8 @@ struct PolPrep {
   double scale = 0.0;
 };
 
-static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
+static gw_status pol_prepare_form(gw_ctx* c, int iq, const double* G, int eform, PolPrep* pp) {
   const int ni = c->ni, nib = (ni + 127) / 128, nb32 = (ni + 31) / 32;
-  // Which form: the producers' X builds pace the E form (one accumulator per build) and the MMAs
-  // the complex form (Re P and Im P from one build). Per (k, tau, chunk), E needs nib ceil(ni / 256)
-  // builds and 3 ni (128 nib) MMA columns, the complex form one build per strip of the Hermitian
-  // half and 6 x its columns; E is the faster one up to ni = 256 (2 builds either way at 256, a
-  // third less MMA work), the complex one above (at 512: 8 builds against 6).
-  const int eform = c->pol_form == 1 ? 1 : c->pol_form == 2 ? 0 : (ni <= 256 ? 1 : 0);
   // strips covering E: rows of block i, columns [0, ni) in pieces <= 256; or covering the upper
   // triangle of P: rows of block i, columns [128 i, ni) in pieces <= 256
   std::vector<int4> strips;
@@ -1065,16 +1059,19 @@ static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
   // the partials of at most pol_part_bytes are held at once: segments run in passes, each
   // reduced into P (the first pass writes, later ones add)
   const size_t seg_bytes = (size_t)base_units * (eform ? 1 : 2) * P_TILE * sizeof(float);  // E form: units of two tau
-  const int seg_pass = (int)std::max<size_t>(1, std::min<size_t>(nseg, c->pol_part_bytes / seg_bytes));
-  const size_t part_bytes = seg_bytes * seg_pass;
+  int seg_pass = (int)std::max<size_t>(1, std::min<size_t>(nseg, c->pol_part_bytes / seg_bytes));
+  if (c->mw.pass_cap) seg_pass = std::min(seg_pass, c->mw.pass_cap);
   const size_t wt_bytes = (size_t)c->nk * c->ntau * npw * sizeof(float);
   const size_t ys_bytes = (size_t)c->nk * cpk * nib * 2 * 128 * 64 * sizeof(__half);
   const size_t xf_bytes = eform ? (size_t)c->nk * cpk * nib * 2 * 128 * 32 * sizeof(float) : 0;
   const size_t e_bytes = eform ? (size_t)c->ntau * ni * ni * sizeof(double) : 0;
   gw_status st;
-  if ((st = ensure(c, &c->mw.wslices, &c->mw.wslices_bytes, part_bytes + wt_bytes + ys_bytes + xf_bytes + e_bytes,
-                   "P workspace")) != GW_OK)
-    return st;
+  // fewer segments per pass where memory is short (remembered: the next call finds its workspace there)
+  while (!grow_ws(c, &c->mw.wslices, &c->mw.wslices_bytes, seg_bytes * seg_pass + wt_bytes + ys_bytes + xf_bytes + e_bytes)) {
+    if (seg_pass == 1 || capturing(c)) return set_err(c, GW_ENOMEM, "tensor-core workspace: P workspace");
+    c->mw.pass_cap = seg_pass /= 2;
+  }
+  const size_t part_bytes = seg_bytes * seg_pass;
   float* d_part = (float*)c->mw.wslices;
   float* d_wt = d_part + part_bytes / sizeof(float);
   __half* d_ys = (__half*)((char*)d_wt + wt_bytes);
@@ -1121,6 +1118,22 @@ static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
   pp->eform = eform;
   pp->scale = 1.0 / ((double)kScaleA * kScaleA * c->omega * c->nk);
   return GW_OK;
+}
+
+static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
+  // Which form: the producers' X builds pace the E form (one accumulator per build) and the MMAs
+  // the complex form (Re P and Im P from one build). Per (k, tau, chunk), E needs nib ceil(ni / 256)
+  // builds and 3 ni (128 nib) MMA columns, the complex form one build per strip of the Hermitian
+  // half and 6 x its columns; E is the faster one up to ni = 256 (2 builds either way at 256, a
+  // third less MMA work), the complex one above (at 512: 8 builds against 6).
+  // The FP32 image XF of the E form doubles the operand bytes; without the memory for it, the complex form runs.
+  if (!c->mw.no_xf && (c->pol_form == 1 || (c->pol_form == 0 && c->ni <= 256))) {
+    const gw_status st = pol_prepare_form(c, iq, G, 1, pp);
+    if (st != GW_ENOMEM || capturing(c)) return st;
+    c->mw.no_xf = true;
+    c->mw.pass_cap = 0;
+  }
+  return pol_prepare_form(c, iq, G, 0, pp);
 }
 
 // Sum the partials of the segments [s0, s0 + ns) into E, then form P from E (the first pass writes
