@@ -264,18 +264,20 @@ __global__ void __launch_bounds__(1024) k_grads(const __grid_constant__ GradJobs
 // ------------------------------------------------------------------ loss and the rest
 // residual R = out A^T - x (FP32), loss = (1/B) sum R^2, dOut = (2/B) R A, dZ = dOut softplus'(Z) of the last
 // layer with its fp16 copies. One block per LS = 8 samples: every element of A is read once for them (one
-// sample where the outputs of eight do not fit in shared memory). 67 -> 24 us at batch 1024.
+// sample, its outputs read from memory, where those of eight do not fit in shared memory). 67 -> 24 us at batch 1024.
 template <int LS>
 __global__ void __launch_bounds__(128) k_loss(const float* __restrict__ out, const float* __restrict__ x,
                                               const float* __restrict__ Acpe, const float* __restrict__ Z, int64_t Bn,
                                               int nout, int nx, float* __restrict__ dZ, __half* __restrict__ dZh,
                                               __half* __restrict__ dZT, float* __restrict__ loss) {
   extern __shared__ float sm[];
-  float* so = sm;               // [nout][LS]
-  float* r = sm + nout * LS;    // [nx][LS]
   const int64_t b0 = (int64_t)blockIdx.x * LS;  // Bn is a multiple of 128
-  for (int e = threadIdx.x; e < nout * LS; e += blockDim.x) so[e] = out[(b0 + e % LS) * nout + e / LS];
-  __syncthreads();
+  const float* so = LS > 1 ? sm : out + b0 * nout;  // [nout][LS]
+  float* r = LS > 1 ? sm + nout * LS : sm;          // [nx][LS]
+  if (LS > 1) {
+    for (int e = threadIdx.x; e < nout * LS; e += blockDim.x) sm[e] = out[(b0 + e % LS) * nout + e / LS];
+    __syncthreads();
+  }
   float part = 0.f;
   for (int i = threadIdx.x; i < nx; i += blockDim.x) {
     float s[LS];
@@ -438,16 +440,16 @@ gw_status backward(gw_mlp* m, int64_t Bn, const float* x, const float* Acpe, int
   gw_status st;
   const int L = m->nlayers, e = L - 1;
   cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream);
-  const size_t sm1 = sizeof(float) * ((size_t)m->nout + nx);
-  auto loss = [&](auto* kernel, int ls) {
-    if (ls * sm1 > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(ls * sm1));
-    kernel<<<(unsigned)(Bn / ls), 128, ls * sm1, m->stream>>>(m->out, x, Acpe, m->Z[e], Bn, m->nout, nx, m->dZ[e], m->dZh[e],
-                                                             m->dZT[e], m->loss);
+  auto loss = [&](auto* kernel, int ls, size_t sm) {
+    if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    kernel<<<(unsigned)(Bn / ls), 128, sm, m->stream>>>(m->out, x, Acpe, m->Z[e], Bn, m->nout, nx, m->dZ[e], m->dZh[e],
+                                                       m->dZT[e], m->loss);
   };
-  if (8 * sm1 <= 200 * 1024)
-    loss(k_loss<8>, 8);
+  const size_t sm8 = 8 * sizeof(float) * ((size_t)m->nout + nx);
+  if (sm8 <= 200 * 1024)
+    loss(k_loss<8>, 8, sm8);
   else
-    loss(k_loss<1>, 1);
+    loss(k_loss<1>, 1, sizeof(float) * nx);
   if ((st = mlp_check(m, "mlp loss")) != GW_OK) return st;
   for (int l = e; l > 0; --l) {  // dZ of the layer below = (dZ W) act'(Z)
     GemmArgs g{m->dZh[l], m->WTh[l], (int)Bn, m->din[l], m->dout[l], nullptr, m->Z[l - 1], m->dZh[l - 1], m->dZT[l - 1],
