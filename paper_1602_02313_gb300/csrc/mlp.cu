@@ -11,6 +11,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -30,8 +31,9 @@ struct gw_mlp {
   float* grads = nullptr;
   std::vector<__half*> Wh, WTh;
   int64_t step = 0;
-  // workspaces for batch <= cap
+  // workspaces for batch <= cap (all of them in `owned`)
   int64_t cap = 0;
+  std::vector<void*> owned;
   std::vector<float*> Z;      // pre-activations [B][dout]
   std::vector<__half*> Hh;    // fp16 activations [B][dout] (layer input of the next)
   std::vector<__half*> HT;    // fp16 transposed activations [dout][B] (incl. input at index 0)
@@ -40,7 +42,7 @@ struct gw_mlp {
   std::vector<float*> dZ;     // per layer [B][dout]
   std::vector<__half*> dZh;   // per layer [B][dout]
   std::vector<__half*> dZT;   // per layer [dout][B]
-  float* part = nullptr;      // [K splits][num_params]: dW over parts of the batch
+  float* part = nullptr;      // [K splits][num_params]: dW over parts of the batch; null: dZ of a layer at a time
   float* loss = nullptr;      // [1]
   int* err = nullptr;
   std::string errmsg;
@@ -378,48 +380,55 @@ gw_status gemm(gw_mlp* m, const GemmArgs& g) {
 // parts of the batch in the dW products: 256 samples each, at most 16 parts
 int dw_part(int64_t Bn) { return (int)std::max<int64_t>(GK, (Bn / 16 + 63) / 64 * 64); }
 
-gw_status ensure_batch(gw_mlp* m, int64_t Bn) {
-  if (Bn <= m->cap) return GW_OK;
-  auto fr = [](void* p) {
-    if (p) cudaFree(p);
+// Workspaces of a batch. Where memory is short (lean), one layer's dZ at a time and no parts of dW: 10 bytes per
+// sample of the widest layer instead of 8 of every layer and up to 16 copies of the parameters.
+bool alloc_batch(gw_mlp* m, int64_t Bn, bool lean) {
+  for (void* p : m->owned) cudaFree(p);
+  m->owned.clear();
+  m->cap = 0;
+  bool ok = true;
+  auto get = [&](auto*& p, size_t n) {
+    p = nullptr;
+    if (ok && (ok = cudaMalloc((void**)&p, sizeof(*p) * n) == cudaSuccess)) m->owned.push_back(p);
   };
   const int L = m->nlayers;
-  for (auto* v : {&m->Z, &m->dZ}) {
-    for (float* p : *v) fr(p);
-    v->assign(L, nullptr);
-  }
-  for (auto* v : {&m->Hh, &m->HT, &m->dZh, &m->dZT}) {
-    for (__half* p : *v) fr(p);
-    v->assign(v == &m->HT ? L + 1 : L, nullptr);
-  }
-  fr(m->Xh);
-  fr(m->out);
-  fr(m->part);
-  m->Xh = nullptr;
-  m->out = m->part = nullptr;
-  bool ok = true;
+  for (auto* v : {&m->Z, &m->dZ}) v->assign(L, nullptr);
+  for (auto* v : {&m->Hh, &m->HT, &m->dZh, &m->dZT}) v->assign(v == &m->HT ? L + 1 : L, nullptr);
+  const size_t widest = (size_t)Bn * *std::max_element(m->dout.begin(), m->dout.end());
+  get(m->HT[0], (size_t)Bn * m->nin);
+  get(m->Xh, (size_t)Bn * m->nin);
+  get(m->out, (size_t)Bn * m->nout);
   for (int l = 0; l < L; ++l) {
     const size_t n = (size_t)Bn * m->dout[l];
-    ok &= cudaMalloc((void**)&m->Z[l], sizeof(float) * n) == cudaSuccess;
-    ok &= cudaMalloc((void**)&m->Hh[l], sizeof(__half) * n) == cudaSuccess;
-    ok &= cudaMalloc((void**)&m->HT[l + 1], sizeof(__half) * n) == cudaSuccess;
-    ok &= cudaMalloc((void**)&m->dZ[l], sizeof(float) * n) == cudaSuccess;
-    ok &= cudaMalloc((void**)&m->dZh[l], sizeof(__half) * n) == cudaSuccess;
-    ok &= cudaMalloc((void**)&m->dZT[l], sizeof(__half) * n) == cudaSuccess;
+    get(m->Z[l], n);
+    get(m->Hh[l], n);
+    get(m->HT[l + 1], n);
+    if (lean && l > 0) {
+      m->dZ[l] = m->dZ[0];
+      m->dZT[l] = m->dZT[0];
+    } else {
+      get(m->dZ[l], lean ? widest : n);
+      get(m->dZT[l], lean ? widest : n);
+    }
+    if (lean && l > 1)
+      m->dZh[l] = m->dZh[l - 2];
+    else
+      get(m->dZh[l], lean ? widest : n);
   }
-  ok &= cudaMalloc((void**)&m->HT[0], sizeof(__half) * Bn * m->nin) == cudaSuccess;
-  ok &= cudaMalloc((void**)&m->Xh, sizeof(__half) * Bn * m->nin) == cudaSuccess;
-  ok &= cudaMalloc((void**)&m->out, sizeof(float) * Bn * m->nout) == cudaSuccess;
+  m->part = nullptr;
   // any batch up to Bn: the number of parts grows with the batch up to 16
-  const int64_t splits = std::min<int64_t>(16, (Bn + GK - 1) / GK);
-  ok &= cudaMalloc((void**)&m->part, sizeof(float) * splits * gw_mlp_num_params(m)) == cudaSuccess;
+  if (!lean) get(m->part, (size_t)std::min<int64_t>(16, (Bn + GK - 1) / GK) * gw_mlp_num_params(m));
   if (!ok) {
     cudaGetLastError();
-    m->cap = 0;
-    return mlp_err(m, GW_ENOMEM, "mlp workspace");
+    return false;
   }
   m->cap = Bn;
-  return GW_OK;
+  return true;
+}
+
+gw_status ensure_batch(gw_mlp* m, int64_t Bn) {
+  if (Bn <= m->cap || alloc_batch(m, Bn, false) || alloc_batch(m, Bn, true)) return GW_OK;
+  return mlp_err(m, GW_ENOMEM, "mlp workspace");
 }
 
 gw_status forward(gw_mlp* m, int64_t Bn, const float* x) {
@@ -435,7 +444,44 @@ gw_status forward(gw_mlp* m, int64_t Bn, const float* x) {
   return GW_OK;
 }
 
-// Gradients into m->grads. More layers than fit the job tables go in runs of kMaxLayers.
+// Gradients of the layers l0 .. l1 - 1 into m->grads, from their dZ. More layers than fit the job tables go in runs of
+// kMaxLayers. Without parts (m->part null) dW is one product over the whole batch, straight into m->grads.
+gw_status weight_grads(gw_mlp* m, int64_t Bn, int l0, int l1) {
+  gw_status st;
+  cudaFuncSetAttribute(k_gemm_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
+  const int64_t np = gw_mlp_num_params(m);
+  const int kpart = m->part ? dw_part(Bn) : (int)Bn, splits = (int)((Bn + kpart - 1) / kpart);
+  float* part = m->part ? m->part : m->grads;
+  for (; l0 < l1; l0 += kMaxLayers) {
+    const int n = std::min(kMaxLayers, l1 - l0);
+    GemmJobs J{};
+    GradJobs D{};
+    J.njobs = D.nlayers = n;
+    J.kpart = kpart;
+    J.stride = D.stride = np;
+    D.splits = splits;
+    D.batch = Bn;
+    for (int i = 0; i < n; ++i) {  // dW = dZ^T H_in : [dout][din], K = batch
+      const int l = l0 + i, d = m->dout[l], di = m->din[l];
+      D.w0[i] = m->gW[l] - m->grads;
+      J.job[i] = GemmArgs{m->dZT[l], m->HT[l], d, di, (int)Bn, nullptr, nullptr, nullptr, nullptr, part + D.w0[i], 0};
+      J.tile0[i + 1] = J.tile0[i] + (d / 128) * (di / GN);
+      D.dZ[i] = m->dZ[l];
+      D.nw[i] = d * di;
+      D.d[i] = d;
+      D.wblk[i] = m->part ? (D.nw[i] + 1023) / 1024 : 0;
+      D.blk0[i + 1] = D.blk0[i] + D.wblk[i] + d / 32;
+    }
+    k_gemm_dw<<<dim3(J.tile0[n], splits), GEMM_THREADS, G_SMEM, m->stream>>>(J, m->err);
+    if ((st = mlp_check(m, "mlp gemm")) != GW_OK) return st;
+    k_grads<<<D.blk0[n], 1024, 0, m->stream>>>(D, m->part, m->grads);
+    if ((st = mlp_check(m, "mlp gradients")) != GW_OK) return st;
+  }
+  return GW_OK;
+}
+
+// Gradients into m->grads: dZ layer by layer downwards, then the weight gradients of all layers in one launch; with one
+// layer's dZ at a time (m->part null) those of a layer before the dZ below it.
 gw_status backward(gw_mlp* m, int64_t Bn, const float* x, const float* Acpe, int nx) {
   gw_status st;
   const int L = m->nlayers, e = L - 1;
@@ -451,40 +497,15 @@ gw_status backward(gw_mlp* m, int64_t Bn, const float* x, const float* Acpe, int
   else
     loss(k_loss<1>, 1, sizeof(float) * nx);
   if ((st = mlp_check(m, "mlp loss")) != GW_OK) return st;
-  for (int l = e; l > 0; --l) {  // dZ of the layer below = (dZ W) act'(Z)
+  for (int l = e; l >= 0; --l) {
+    if (!m->part && (st = weight_grads(m, Bn, l, l + 1)) != GW_OK) return st;
+    if (l == 0) break;
+    // dZ of the layer below = (dZ W) act'(Z)
     GemmArgs g{m->dZh[l], m->WTh[l], (int)Bn, m->din[l], m->dout[l], nullptr, m->Z[l - 1], m->dZh[l - 1], m->dZT[l - 1],
                m->dZ[l - 1], 0};
     if ((st = gemm<EPI_BACK>(m, g)) != GW_OK) return st;
   }
-  cudaFuncSetAttribute(k_gemm_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
-  const int64_t np = gw_mlp_num_params(m);
-  const int kpart = dw_part(Bn), splits = (int)((Bn + kpart - 1) / kpart);
-  for (int l0 = 0; l0 < L; l0 += kMaxLayers) {
-    const int n = std::min(kMaxLayers, L - l0);
-    GemmJobs J{};
-    GradJobs D{};
-    J.njobs = D.nlayers = n;
-    J.kpart = kpart;
-    J.stride = D.stride = np;
-    D.splits = splits;
-    D.batch = Bn;
-    for (int i = 0; i < n; ++i) {  // dW = dZ^T H_in : [dout][din], K = batch
-      const int l = l0 + i, d = m->dout[l], di = m->din[l];
-      D.w0[i] = m->gW[l] - m->grads;
-      J.job[i] = GemmArgs{m->dZT[l], m->HT[l], d, di, (int)Bn, nullptr, nullptr, nullptr, nullptr, m->part + D.w0[i], 0};
-      J.tile0[i + 1] = J.tile0[i] + (d / 128) * (di / GN);
-      D.dZ[i] = m->dZ[l];
-      D.nw[i] = d * di;
-      D.d[i] = d;
-      D.wblk[i] = (D.nw[i] + 1023) / 1024;
-      D.blk0[i + 1] = D.blk0[i] + D.wblk[i] + d / 32;
-    }
-    k_gemm_dw<<<dim3(J.tile0[n], splits), GEMM_THREADS, G_SMEM, m->stream>>>(J, m->err);
-    if ((st = mlp_check(m, "mlp gemm")) != GW_OK) return st;
-    k_grads<<<D.blk0[n], 1024, 0, m->stream>>>(D, m->part, m->grads);
-    if ((st = mlp_check(m, "mlp gradients")) != GW_OK) return st;
-  }
-  return GW_OK;
+  return m->part ? weight_grads(m, Bn, 0, L) : GW_OK;
 }
 
 gw_status refresh_half(gw_mlp* m) {
@@ -605,14 +626,12 @@ gw_status gw_mlp_destroy(gw_mlp* m) {
   auto fr = [](void* p) {
     if (p) cudaFree(p);
   };
-  for (auto* v : {&m->W, &m->b, &m->mW, &m->vW, &m->mb, &m->vb, &m->Z, &m->dZ})
+  for (auto* v : {&m->W, &m->b, &m->mW, &m->vW, &m->mb, &m->vb})
     for (float* p : *v) fr(p);
-  for (auto* v : {&m->Wh, &m->WTh, &m->Hh, &m->HT, &m->dZh, &m->dZT})
+  for (auto* v : {&m->Wh, &m->WTh})
     for (__half* p : *v) fr(p);
+  for (void* p : m->owned) fr(p);
   fr(m->grads);
-  fr(m->part);
-  fr(m->Xh);
-  fr(m->out);
   fr(m->loss);
   fr(m->err);
   delete m;
