@@ -34,6 +34,8 @@ struct gw_mlp {
   // workspaces for batch <= cap (all of them in `owned`)
   int64_t cap = 0;
   std::vector<void*> owned;
+  bool captured = false;       // a call was captured into a graph: outgrown workspaces are kept, in `retired`
+  std::vector<void*> retired;
   std::vector<float*> Z;      // pre-activations [B][dout]
   std::vector<__half*> Hh;    // fp16 activations [B][dout] (layer input of the next)
   std::vector<__half*> HT;    // fp16 transposed activations [dout][B] (incl. input at index 0)
@@ -383,7 +385,10 @@ int dw_part(int64_t Bn) { return (int)std::max<int64_t>(GK, (Bn / 16 + 63) / 64 
 // Workspaces of a batch. Where memory is short (lean), one layer's dZ at a time and no parts of dW: 10 bytes per
 // sample of the widest layer instead of 8 of every layer and up to 16 copies of the parameters.
 bool alloc_batch(gw_mlp* m, int64_t Bn, bool lean) {
-  for (void* p : m->owned) cudaFree(p);
+  if (m->captured)
+    m->retired.insert(m->retired.end(), m->owned.begin(), m->owned.end());
+  else
+    for (void* p : m->owned) cudaFree(p);
   m->owned.clear();
   m->cap = 0;
   bool ok = true;
@@ -420,6 +425,8 @@ bool alloc_batch(gw_mlp* m, int64_t Bn, bool lean) {
   if (!lean) get(m->part, (size_t)std::min<int64_t>(16, (Bn + GK - 1) / GK) * gw_mlp_num_params(m));
   if (!ok) {
     cudaGetLastError();
+    for (void* p : m->owned) cudaFree(p);
+    m->owned.clear();
     return false;
   }
   m->cap = Bn;
@@ -427,6 +434,12 @@ bool alloc_batch(gw_mlp* m, int64_t Bn, bool lean) {
 }
 
 gw_status ensure_batch(gw_mlp* m, int64_t Bn) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(m->stream, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    cs = cudaStreamCaptureStatusActive;
+  }
+  if (cs != cudaStreamCaptureStatusNone) m->captured = true;
   if (Bn <= m->cap || alloc_batch(m, Bn, false) || alloc_batch(m, Bn, true)) return GW_OK;
   return mlp_err(m, GW_ENOMEM, "mlp workspace");
 }
@@ -631,6 +644,7 @@ gw_status gw_mlp_destroy(gw_mlp* m) {
   for (auto* v : {&m->Wh, &m->WTh})
     for (__half* p : *v) fr(p);
   for (void* p : m->owned) fr(p);
+  for (void* p : m->retired) fr(p);
   fr(m->grads);
   fr(m->loss);
   fr(m->err);

@@ -78,3 +78,34 @@ def test_replay_after_a_larger_call(name):
         assert all(bool(torch.isfinite(torch.view_as_real(r)).all()) and torch.equal(o, r) for o, r in zip(out, ref))
         ctx.sync()
     ctx.close()
+
+
+def test_seed_network_replay_after_a_larger_batch():
+    import torch
+
+    import paper_1602_02313_gb300 as gw
+    from paper_1602_02313_gb300 import build as b
+    b.build()
+    rng = np.random.default_rng(18)
+    x = torch.from_numpy(rng.standard_normal((1024, 64)).astype(np.float32)).cuda()
+    A = torch.from_numpy((0.1 * rng.standard_normal((64, 128))).astype(np.float32)).cuda()
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(st):
+        net = gw.MLP(nin=64, nh=128, nhidden=2, nout=128, seed=2, stream=st)
+        loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+        g1, g2 = (torch.zeros(net.num_params(), dtype=torch.float32, device="cuda") for _ in range(2))
+        net.loss_grad(x[:128], A, loss, g1)
+        st.synchronize()
+        ref = g1.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            net.loss_grad(x[:128], A, loss, g1)
+        net.loss_grad(x, A, loss, g2)
+        st.synchronize()
+        g1.fill_(float("nan"))
+        graph.replay()
+        st.synchronize()
+        assert bool(torch.isfinite(ref).all()) and torch.equal(g1, ref)
+        net.sync()
+    net.close()
