@@ -385,8 +385,9 @@ gw_status launch_bose_exact(gw_ctx* c, int dir, int count, int64_t batch, const 
   // M tiles (of 128 rows; backward: pairs of them) in all and per piece: whole waves within kPiece
   const int64_t tiles = fwd ? (batch * count + 127) / 128 : (int64_t)per_z * count;
   const size_t tile_bytes = (size_t)(fwd ? 1 : 2) * chunks * XA_BYTES;
-  const int64_t waves = std::max<int64_t>(1, (int64_t)(kPiece / tile_bytes) / 152);
-  const int per = (int)std::min<int64_t>(tiles, waves * 152);
+  const int sms = num_sms(c);
+  const int64_t waves = std::max<int64_t>(1, (int64_t)(kPiece / tile_bytes) / sms);
+  const int per = (int)std::min<int64_t>(tiles, waves * sms);
   const size_t b_ea = align256(4 * 256 * (size_t)per);
   if (!x_workspace(c, XW_BOSE, b_ea + (size_t)per * tile_bytes)) return GW_EUNSUPPORTED;
   int* ea = (int*)c->x_ws[XW_BOSE];

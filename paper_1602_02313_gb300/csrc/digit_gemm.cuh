@@ -380,9 +380,7 @@ template <class OP>
 gw_status run_gemm(gw_ctx* c, const typename OP::Job& J, int nunits, const char* what) {
   const size_t smem = 1024 + X_ST * XST_BYTES + sizeof(XSmem);
   cudaFuncSetAttribute(k_digit_gemm<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  if (sms < 1) sms = 148;
+  const int sms = num_sms(c);
   k_digit_gemm<OP><<<nunits < sms ? nunits : sms, X_THREADS, smem, c->stream>>>(J, nunits, c->d_err, c->wait_cycles,
                                                                                 c->fault_stall);
   return check_launch(c, what);

@@ -284,7 +284,7 @@ gw_status launch_offdiag_digits(gw_ctx* c, int iq, const double* G, const double
   const size_t left = kOdBudget > bytes_w(tg) ? kOdBudget - bytes_w(tg) : 0;
   const int kg = (int)std::max<size_t>(1, std::min<size_t>(nk, left / bytes_k(tg)));
   const int tiles2 = kg * mt2(tg) * nt2;
-  const int nsplit = std::max(1, std::min({304 / tiles2, ch2 / (2 * X_BLK), 16}));
+  const int nsplit = std::max(1, std::min({2 * num_sms(c) / tiles2, ch2 / (2 * X_BLK), 16}));
   const size_t b_ew = align256(sizeof(int) * (size_t)ntau * ni), b_w = align256(bytes_w(tg)),
                b_max = align256(4 * ((size_t)kg * np + (size_t)kg * nb + (size_t)kg * (tg + x) * nb)),
                b_a = align256((size_t)mt1(kg) * ch1 * XA_BYTES), b_b = align256((size_t)kg * nt2 * ch2 * XB_BYTES),

@@ -423,11 +423,12 @@ gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P) {
   tg = (ntau + (ntau + tg - 1) / tg - 1) / ((ntau + tg - 1) / tg);  // groups of equal size
   const int mt = mtiles(tg);
   // K splits: whole accumulation blocks, as many as give the least waves x (chunks + a unit's fixed cost)
+  const int sms = num_sms(c);
   int nsplit = 1;
   double best = 1e300;
   for (int s = 1; s <= std::min(64, (nc + X_BLK - 1) / X_BLK); ++s) {
     const int L = (nc + s - 1) / s, units = mt * nt * s;
-    const double t = (double)((units + 151) / 152) * (L + 8.0);
+    const double t = (double)((units + sms - 1) / sms) * (L + 8.0);
     if (t < best * 0.98) {
       best = t;
       nsplit = s;
@@ -467,7 +468,7 @@ gw_status launch_pol_exact(gw_ctx* c, int iq, const double* G, double* P) {
     for (int t0 = 0; t0 < ntau; t0 += tg) {
       const int tn = std::min(tg, ntau - t0);
       const int64_t ns = ((int64_t)cn * ni + 255) / 256;  // blocks; several tau per thread once they fill the GPU
-      const int tpt = (int)std::max<int64_t>(1, std::min<int64_t>(tn, ns * tn / 1216));
+      const int tpt = (int)std::max<int64_t>(1, std::min<int64_t>(tn, ns * tn / (8 * sms)));
       k_xslice_pol<<<dim3((unsigned)ns, (tn + tpt - 1) / tpt), 256, 0, c->stream>>>(M, w, ey, ex, nk, ni, np, c0, cn, t0, tn,
                                                                                   tpt, t0 == 0, Yi, Xi);
       if ((st = check_launch(c, "exact pol digits")) != GW_OK) return st;

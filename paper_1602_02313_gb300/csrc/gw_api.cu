@@ -519,6 +519,12 @@ __global__ void k_sigx_occ(const double* __restrict__ vm, const int* __restrict_
   Sx[e] += pref * s;
 }
 
+int num_sms(const gw_ctx* c) {
+  int n = 0;
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, c->device);
+  return n > 0 ? n : 152;
+}
+
 bool capturing(gw_ctx* c) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) {

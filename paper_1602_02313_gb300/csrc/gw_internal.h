@@ -145,6 +145,7 @@ gw_status check_launch(gw_ctx* c, const char* what);
 void kt_begin(gw_ctx* c, const char* name);
 void kt_end(gw_ctx* c);
 gw_status set_err(gw_ctx* c, gw_status s, const std::string& msg);
+int num_sms(const gw_ctx* c);
 // whether the context's stream is being captured (or may be); remembered in c->captured
 bool capturing(gw_ctx* c);
 // Makes the workspace *p of *have bytes hold at least `need`; false when the memory cannot be had (*p is then

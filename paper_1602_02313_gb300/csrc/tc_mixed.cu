@@ -1009,12 +1009,6 @@ gw_status ensure(gw_ctx* c, void** p, size_t* have, size_t need, const char* wha
   return GW_OK;
 }
 
-int num_sms(gw_ctx* c) {
-  int n = 0;
-  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, c->device);
-  return n > 0 ? n : 148;
-}
-
 }  // namespace
 
 // Host plan of one polarization job: strips, K segments, workspace, and the operand image and
