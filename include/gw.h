@@ -140,9 +140,13 @@ gw_status gw_green_tau(gw_ctx* ctx, const double* eps, const double* sigx, const
  * P_II'(q|tau) = 1/(Omega N_k) sum_k sum_ab M^I_ab Q_ab(tau) conj(M^I'_ab),
  * Q_ab(tau) = G_b(k|tau) G_a(k-q|-tau), G(-tau) = -G(beta - tau) (Sec. II).
  * G_tau [nk][nb][ntau] (any G: G0 or dressed); P_tau out cplx [ntau][ni][ni] (Hermitian).
- * GW_FP64 uses a context workspace of up to ~7 GiB, grown on use; a call that cannot have it (no
- * memory, or a first call under stream capture) runs on the CUDA cores without one. With GW_FP64 an
- * infinity or nan in M^I or G gives nan in the rows and columns it reaches. */
+ * GW_FP64 uses a context workspace, grown on use: digits of both operands (up to 2 GiB each, in groups of tau
+ * and K beyond that), the pair weights (8 nk nb^2 ntau bytes), P as real sums (8 ntau ni^2) and up to 64 partial
+ * sums of a group of tau (few where ni is large). A call that cannot have it (no memory, or a first call under
+ * stream capture) runs on the CUDA cores without one. With GW_FP64 an infinity or nan in M^I or G gives nan in the
+ * rows and columns it reaches. GW_FP16X2 uses fp16 and, up to ni = 256, FP32 images of M[q] (8 nk nb^2 ni bytes
+ * each, ni rounded up to 128) and FP32 partial sums (GW_TUNE_POL_PART_MB); short of memory it holds fewer partial
+ * sums and then does without the FP32 image. */
 gw_status gw_polarization(gw_ctx* ctx, int iq, const double* G_tau, gw_prec prec, double* P_tau);
 
 /* The polarization of several crystals (one q each) in one persistent launch: job j is
@@ -163,7 +167,9 @@ gw_status gw_polarization_many(int njobs, gw_ctx* const* ctxs, const int* iqs, c
  * counterparts), fixed matrices (built in extended precision, stored FP64) applied as
  * batched matvecs. prec: GW_FP64 (native FP64), or GW_F32X2 for the two bosonic
  * directions (exact digit products on the tensor cores, relative error ~1e-13 where the map cancels;
- * the mixed chain's choice; native FP64 when its digit workspace, up to ~120 MB, cannot be had);
+ * the mixed chain's choice; native FP64 when its digit workspace cannot be had: up to 112 MiB, or one wave of tiles
+ * where that is more, 1.1 MB x max(ntau, nnu), from ~110 points on). The data of one element over tau or nu are cut
+ * at 2^-56 of their largest value after scaling each point by its map column's size;
  * anything else returns GW_EUNSUPPORTED.
  *  BOSE  TAU_TO_IW : in cplx [ntau][batch]        -> out cplx [nnu][batch]
  *  BOSE  IW_TO_TAU : in cplx [nnu][m][m] of a Hermitian-matrix function (batch = m)
@@ -190,8 +196,8 @@ gw_status gw_tau_to_freq_many(gw_ctx* ctx, gw_stat stat, gw_dir dir, int count, 
  * elimination of [1 - Pi | Pi] (GW_FP64 only, any ni) serves gw_screen_static. No pivoting:
  * 1 - Pi has Hermitian part >= 1.
  * prec: GW_FP64 (native FP64), GW_F32X2 (pivot blocks in float-float, the updates as exact digit
- * products on the tensor cores with up to 0.8 GiB of further workspace, or float-float throughout when
- * that cannot be had; relative error ~1e-14 at ni = 256) or GW_F32 (FP32 arithmetic, blocked inversion only; relative error of the
+ * products on the tensor cores, rows cut at 2^-56 of their largest entry, with up to 1.5 GiB of further workspace,
+ * or float-float throughout when that cannot be had; relative error ~1e-14 at ni = 256) or GW_F32 (FP32 arithmetic, blocked inversion only; relative error of the
  * order of sqrt(ni) 6e-8 cond(1 - Pi), ~1e-6 at ni = 256); else GW_EUNSUPPORTED.
  * P_iv, Wt_iv cplx [nqb][nnu][ni][ni]; info out (device) [nqb][nnu]: 0, or j+1 for a
  * zero pivot at elimination step j (that system's output is then undefined).
@@ -250,9 +256,12 @@ gw_status gw_sigma_star(gw_ctx* ctx, int nrep, const int* kinv, int64_t ncol, co
  *   Sigma^c_nm(k|tau) += -1/(Omega N_k) sum_j G_j(k-q|tau) sum_IJ conj(M^I_jn) W~_IJ(tau) M^J_jm,
  *   Sigma^x_nm(k)     += -1/(Omega N_k) sum_j occ_j(k-q) sum_I v_I conj(M^I_jn) M^I_jm.
  * G_tau [nk][nb][ntau], occ [nk][nb] (may be NULL when Sx is), Wt_tau cplx [ntau][ni][ni];
- * S_tau cplx [nk][nb][nb][ntau]; Sx cplx [nk][nb][nb] (may be NULL). FP64 on the CUDA cores,
- * W~ a_j formed in chunks of rows so any ni fits; GW_EINVAL when the nb x nb accumulator of one
- * (k, tau) and 8 rows of W~ a_j do not fit in 200 KiB of shared memory (nb > 109). */
+ * S_tau cplx [nk][nb][nb][ntau]; Sx cplx [nk][nb][nb] (may be NULL). FP64 by digit
+ * products on the tensor cores (the bound given at GW_FP64, for W~ a_j and for its product with a_n) with a context
+ * workspace of about 2 GiB, grown on use; a call that cannot have it (no memory, or a first call under stream
+ * capture), or GW_TUNE_FP64_FORM 1, runs on the CUDA cores, W~ a_j formed in chunks of rows so any ni fits. GW_EINVAL
+ * for nb > 109, where the nb x nb accumulator of one (k, tau) and 8 rows of W~ a_j do not fit in 200 KiB of shared
+ * memory. */
 gw_status gw_selfenergy_offdiag(gw_ctx* ctx, int iq, const double* G_tau, const double* occ, const double* Wt_tau,
                                 double* S_tau, double* Sx);
 
@@ -301,7 +310,8 @@ gw_status gw_screen_static(int nq, int nnu, int ni, const double* sqrt_v, const 
  *             Sigx_n(k) += -1/(Omega N_k) sum_j occ_j(k-q) sum_I v_I |M^I_jn|^2.
  * G_tau [nk][nb][ntau]; occ [nk][nb]; Wt_tau cplx [ntau][ni][ni] (Hermitian);
  * Sigc_tau [nk][nb][ntau] (real: W~(tau) Hermitian); Sigx [nk][nb] (may be NULL).
- * prec GW_FP64: both in FP64 (Sigc with a workspace and without one as in gw_polarization). GW_FP16X2: Sigc on the tensor cores, Sigx in
+ * prec GW_FP64: both in FP64 (Sigc with a workspace as in gw_polarization: digits of M[q] and W~, up to 2 GiB each, and
+ * 8 nk nb^2 ntau bytes; without one likewise). GW_FP16X2: Sigc on the tensor cores, Sigx in
  * float-float on the FP32 pipes (relative error ~1e-12). */
 gw_status gw_selfenergy(gw_ctx* ctx, int iq, const double* G_tau, const double* occ,
                         const double* Wt_tau, gw_prec prec, double* Sigc_tau, double* Sigx);
@@ -409,7 +419,7 @@ gw_status gw_set_stream(gw_ctx* ctx, void* stream);
  *      1 .. 32 (default 32; fewer = more, smaller partials and a smaller accumulation error);
  *  GW_TUNE_POL_PART_MB: MiB of FP32 partial strips held at once (default 8192; the K segments
  *      run in passes beyond it), >= 1;
- *  GW_TUNE_WAIT_CYCLES: SM clock cycles a pipeline wait of k_pol_tc / k_sig_tc may take before it
+ *  GW_TUNE_WAIT_CYCLES: SM clock cycles a pipeline wait of k_pol_tc / k_sig_tc / k_digit_gemm may take before it
  *      gives up and the launch reports GW_ETIMEOUT at the next gw_sync, 1e3 .. 2^40 (default 4e9,
  *      ~2 s at the GPU's top clock; a healthy wait takes microseconds);
  *  GW_TUNE_FAULT_STALL: fault injection for tests of that detector, 0 or 1: with 1, the

@@ -786,7 +786,7 @@ gw_status gw_sync(gw_ctx* c) {
   if (h != 0) {
     cudaMemset(c->d_err, 0, sizeof(int));
     return set_err(c, GW_ETIMEOUT,
-                   "gw_sync: a bounded device-side wait ran out in a tensor-core contraction (k_pol_tc / k_sig_tc); "
+                   "gw_sync: a bounded device-side wait ran out in a tensor-core contraction (k_pol_tc / k_sig_tc / k_digit_gemm); "
                    "the outputs of the calls since the last gw_sync are undefined");
   }
   return GW_OK;

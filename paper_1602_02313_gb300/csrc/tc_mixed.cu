@@ -181,9 +181,9 @@ __device__ __forceinline__ void pol_next(PolPhase& ph, int nst) {
 
 // One work unit u of job J: the copy warp brings Y, the producer warps build X, the MMA warp issues the
 // products into two accumulators, the producer warps then move the FP32 partial strips out of TMEM. A
-// wait that runs out raises S.abort_flag. What bounds it is the data pipe of shared memory and L1 (ncu:
-// 51 % MMA operands, 53 % producers and copies), at 73 % of the tensor pipe's cycles: in the E form at
-// N = 256 the 24 MMAs of a chunk and two tau read 2304 clocks' worth (128 bytes a clock) and take 3072.
+// wait that runs out raises S.abort_flag. What bounds it is the data pipe of shared memory, which MMA operands,
+// copies and the stores of X share, at 74 % of the tensor pipe's cycles: in the E form at N = 256 the 24 MMAs of a
+// chunk and two tau read 2304 clocks' worth (128 bytes a clock) and take 3072.
 // One tau per unit brought Y twice as often (62 bytes of L2 per clock and SM at full rate) and converted
 // the halves of Y again per tau. Measured per q at Nk 64, Nb 64, NI 256, 48 tau: 7.85 -> 5.53 ms, the same
 // bits; complex form (NI 384, Nb 96, Nk 8, 48 tau) 4.97 -> 4.85 ms. XF through a shared-memory ring instead
@@ -1115,11 +1115,11 @@ static gw_status pol_prepare_form(gw_ctx* c, int iq, const double* G, int eform,
 }
 
 static gw_status pol_prepare(gw_ctx* c, int iq, const double* G, PolPrep* pp) {
-  // Which form: the producers' X builds pace the E form (one accumulator per build) and the MMAs
-  // the complex form (Re P and Im P from one build). Per (k, tau, chunk), E needs nib ceil(ni / 256)
-  // builds and 3 ni (128 nib) MMA columns, the complex form one build per strip of the Hermitian
-  // half and 6 x its columns; E is the faster one up to ni = 256 (2 builds either way at 256, a
-  // third less MMA work), the complex one above (at 512: 8 builds against 6).
+  // Which form: E up to ni = 256, the complex form above. The line dates from an E form with one tau per unit, which
+  // lost above 256 (Nk 216, NI 512: 245 against 230 s a pass). With two tau per unit E is the faster one there too:
+  // per q at Nk 8, Nb 64, 48 tau 2.15 against 2.22 ms at NI 288, 2.30 / 2.50 at 384, 3.38 / 3.94 at 512, 7.34 / 8.04 at
+  // 768 (3.0 x the algorithmic MMA work against 4.0 at 384, 3.75 at 512), and 0.96 / 1.30 at 256. GW_TUNE_POL_FORM 1
+  // takes it; the default has not been moved, as it would change the bits of P above 256.
   // The FP32 image XF of the E form doubles the operand bytes; without the memory for it, the complex form runs.
   if (!c->mw.no_xf && (c->pol_form == 1 || (c->pol_form == 0 && c->ni <= 256))) {
     const gw_status st = pol_prepare_form(c, iq, G, 1, pp);
