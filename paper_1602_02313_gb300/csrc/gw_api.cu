@@ -178,7 +178,8 @@ const double* m_block(gw_ctx* c, int iq) {
     return c->d_M + 2 * (size_t)iq * per_q;
   }
   if (!c->m_per_q) return c->d_M + 2 * (size_t)iq * per_q;
-  if (c->m_cur != iq) {
+  capturing(c);  // a captured call generates its own block at its replays: m_cur is no longer the device's state then
+  if (c->captured || c->m_cur != iq) {
     k_gen_m<<<152 * 8, 256, 0, c->stream>>>((double2*)c->d_M_own, per_q, (uint64_t)(c->q0 + iq) * per_q, c->seed,
                                              std::sqrt(0.5 / c->nb));
     if (check_launch(c, "gen_m") != GW_OK) {

@@ -117,7 +117,8 @@ struct gw_ctx {
   void* x_ws[5] = {};           // digit products on the tensor cores: operand digits, partial sums
   size_t x_ws_bytes[5] = {};
   void* d_bdig = nullptr;       // digits of the bosonic maps (digit_bose.cu)
-  bool captured = false;        // a call was captured into a graph, which keeps the workspaces it saw
+  bool captured = false;        // a call was captured into a graph: it keeps the workspaces it saw, and its replays
+                                // change what is staged there without the host's knowing (mw.iq, m_cur)
   std::vector<void*> retired;   // workspaces outgrown since: freed with the context
   // tensor-core path
   gwi::MixedWork mw;

@@ -1241,7 +1241,9 @@ gw_status launch_sigma_mixed(gw_ctx* c, int iq, const double* G, const double* W
   __half* WS = XS + xbytes / sizeof(__half);
   double* D = (double*)((char*)c->mw.mslices + xbytes + wbytes);
   float2* XE = (float2*)((char*)D + dbytes);
-  if (c->mw.iq != iq || c->mw.prec != prec) {
+  // XS holds the last executed call's q; a captured call executes at its replays, so that it brings its own and the
+  // host's record is no longer the device's state
+  if (c->captured || c->mw.iq != iq || c->mw.prec != prec) {
     const double2* Mq = (const double2*)m_block(c, iq);
     if (!Mq) return GW_ECUDA;
     dim3 g(npp / 32, (c->ni + SX_I - 1) / SX_I, c->nk);
