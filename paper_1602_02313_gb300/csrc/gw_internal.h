@@ -37,10 +37,8 @@ struct MixedWork {
   size_t mslices_bytes = 0;
   void* wslices = nullptr;    // per-tau split copies of W~ (Sigma) or scaled rows (P)
   size_t wslices_bytes = 0;
-  double* dacc = nullptr;     // P strip metadata (uploaded once per context) and error word
-  size_t dacc_bytes = 0;
-  bool strips_ready = false;
-  int strips_form = -1;       // the form the uploaded strips were built for
+  void* strips[2] = {};       // strips of P, by form (complex, E): uploaded at the first call of each and not changed
+  size_t strips_bytes[2] = {};
   int pass_cap = 0;           // memory was short: at most this many K segments of P per pass (0: no limit)
   bool no_xf = false;         // memory was short for the E form of P at one segment per pass
 };

@@ -1072,18 +1072,19 @@ static gw_status pol_prepare_form(gw_ctx* c, int iq, const double* G, int eform,
   float* d_xf = (float*)((char*)d_ys + ys_bytes);
   double* d_e = (double*)((char*)d_xf + xf_bytes);
   const size_t meta_bytes = sizeof(int4) * strips.size() + sizeof(int) * strip_of.size();
-  const void* meta_before = c->mw.dacc;
-  if ((st = ensure(c, (void**)&c->mw.dacc, &c->mw.dacc_bytes, meta_bytes + 256, "P strips")) != GW_OK) return st;
-  if (c->mw.dacc != meta_before || c->mw.strips_form != eform) c->mw.strips_ready = false;
-  int4* d_strips = reinterpret_cast<int4*>(c->mw.dacc);
+  const bool fresh = !c->mw.strips[eform];  // depends on ni and the form only
+  if ((st = ensure(c, &c->mw.strips[eform], &c->mw.strips_bytes[eform], meta_bytes + 256, "P strips")) != GW_OK) return st;
+  int4* d_strips = reinterpret_cast<int4*>(c->mw.strips[eform]);
   int* d_strip_of = reinterpret_cast<int*>(d_strips + strips.size());
-  if (!c->mw.strips_ready) {  // depends on ni and the form: uploaded on the first call of each
+  if (fresh) {
     if (cudaMemcpy(d_strips, strips.data(), sizeof(int4) * strips.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         (!strip_of.empty() && cudaMemcpy(d_strip_of, strip_of.data(), sizeof(int) * strip_of.size(),
-                                         cudaMemcpyHostToDevice) != cudaSuccess))
+                                         cudaMemcpyHostToDevice) != cudaSuccess)) {
+      cudaFree(c->mw.strips[eform]);
+      c->mw.strips[eform] = nullptr;
+      c->mw.strips_bytes[eform] = 0;
       return set_err(c, GW_ECUDA, "P strips upload");
-    c->mw.strips_ready = true;
-    c->mw.strips_form = eform;
+    }
   }
   // rows >= ni of the last block stay as they are: they reach only rows of the strips that nothing reads
   const double2* Mq = (const double2*)m_block(c, iq);
@@ -1273,7 +1274,8 @@ gw_status launch_sigma_mixed(gw_ctx* c, int iq, const double* G, const double* W
 void free_mixed(gw_ctx* c) {
   if (c->mw.mslices) cudaFree(c->mw.mslices);
   if (c->mw.wslices) cudaFree(c->mw.wslices);
-  if (c->mw.dacc) cudaFree(c->mw.dacc);
+  for (void* p : c->mw.strips)
+    if (p) cudaFree(p);
   c->mw = MixedWork();
 }
 

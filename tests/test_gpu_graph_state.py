@@ -86,3 +86,42 @@ def test_polarization_with_generated_elements(prec):
     P = torch.zeros(NT, 64, 64, dtype=torch.complex128, device="cuda")
     torch.cuda.synchronize()
     _check(torch, st, ctx, lambda q: ctx.polarization(q, G, P, gw.PREC[prec]), P)
+
+
+@pytest.mark.parametrize("first,second", [(1, 2), (2, 1)])
+def test_polarization_forms(first, second):
+    """A graph of one form of P replays to the same bits after eager calls of the other, whose strips differ."""
+    import torch
+
+    import paper_1602_02313_gb300 as gw
+    from paper_1602_02313_gb300 import build as b
+    b.build()
+    cr = gi.make_crystal(32, 2, 8, 4, 160, 30.0, qlist=[1])
+    gr = gi.make_grid(30.0, NT, NT, NT, ncont=16)
+    G, _ = orc.green_tau0(cr.eps, gr.tau, gr.beta)
+    Gd = torch.from_numpy(G).cuda()
+    P = torch.zeros(NT, 160, 160, dtype=torch.complex128, device="cuda")
+    st = torch.cuda.Stream()
+    ctx = gw.GW(gr, cr, stream=st, m_mode=1)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        ref = {}
+        for form in (first, second, first):
+            ctx.set_tuning(gw.GW_TUNE_POL_FORM, form)
+            ctx.polarization(0, Gd, P, gw.GW_FP16X2)
+            st.synchronize()
+            assert form not in ref or torch.equal(ref[form], P)
+            ref[form] = P.clone()
+        assert not torch.equal(ref[first], ref[second])
+        g = _capture(torch, st, lambda: ctx.polarization(0, Gd, P, gw.GW_FP16X2))
+        for form in (second, first):
+            ctx.set_tuning(gw.GW_TUNE_POL_FORM, form)
+            ctx.polarization(0, Gd, P, gw.GW_FP16X2)
+            st.synchronize()
+            assert torch.equal(P, ref[form])
+            P.fill_(float("nan"))
+            g.replay()
+            st.synchronize()
+            assert torch.equal(P, ref[first])
+        ctx.sync()
+    ctx.close()
