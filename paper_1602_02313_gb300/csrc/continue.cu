@@ -762,7 +762,10 @@ extern "C" gw_status gw_cpe_setup(gw_ctx* c, int ng, const double* x, double rid
     }
   for (double** p : {&c->d_cpe_x, &c->d_cpe_A, &c->d_cpe_N, &c->d_cpe_tab})
     if (*p) {
-      cudaFree(*p);
+      if (c->captured)
+        c->retired.push_back(*p);  // a captured gw_continue replays with the grid it saw
+      else
+        cudaFree(*p);
       *p = nullptr;
     }
   if (cudaMalloc((void**)&c->d_cpe_x, sizeof(double) * (ng + 2)) != cudaSuccess ||
@@ -786,6 +789,7 @@ extern "C" gw_status gw_cpe_setup(gw_ctx* c, int ng, const double* x, double rid
 extern "C" gw_status gw_cpe_coeffs(gw_ctx* c, double* b) {
   if (!c || !b || !c->d_cpe_b || c->cpe_nprob <= 0) return GW_EINVAL;
   const size_t bytes = (size_t)c->cpe_nprob * c->cpe_ngrid * sizeof(double);
+  capturing(c);  // a captured copy keeps its source
   if (cudaMemcpyAsync(b, c->d_cpe_b, bytes, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
     return set_err(c, GW_ECUDA, "gw_cpe_coeffs");
   return GW_OK;
@@ -840,6 +844,7 @@ extern "C" gw_status gw_cpe_features(gw_ctx* c, int64_t nprob, const double* sig
 extern "C" gw_status gw_cpe_fit_matrix(gw_ctx* c, int nfit, float* A) {
   if (!c || !A || c->cpe_ngrid == 0 || nfit < 1 || nfit > c->ncont) return GW_EINVAL;
   const int n = 2 * nfit * c->cpe_ngrid;
+  capturing(c);  // a captured call keeps its grid
   k_cpe_fitmat<<<(n + 255) / 256, 256, 0, c->stream>>>(c->d_cpe_A, c->ncont, c->cpe_ngrid, nfit, A);
   return check_launch(c, "cpe_fit_matrix");
 }
@@ -856,6 +861,7 @@ extern "C" gw_status gw_cpe_seed(gw_ctx* c, int64_t nprob, const float* bhat, co
 
 extern "C" gw_status gw_cpe_iterations(gw_ctx* c, int* iters) {
   if (!c || !iters || !c->d_cpe_iters || c->cpe_nprob <= 0) return GW_EINVAL;
+  capturing(c);  // a captured copy keeps its source
   if (cudaMemcpyAsync(iters, c->d_cpe_iters, c->cpe_nprob * sizeof(int), cudaMemcpyDeviceToDevice, c->stream) !=
       cudaSuccess)
     return set_err(c, GW_ECUDA, "gw_cpe_iterations");

@@ -109,3 +109,47 @@ def test_seed_network_replay_after_a_larger_batch():
         assert bool(torch.isfinite(ref).all()) and torch.equal(g1, ref)
         net.sync()
     net.close()
+
+
+def test_continuation_replay_after_another_grid():
+    """A captured continuation keeps its pole grid: another gw_cpe_setup and a larger fit after it, then the replay."""
+    import torch
+
+    import paper_1602_02313_gb300 as gw
+    from paper_1602_02313_gb300 import build as b
+    from paper_1602_02313_gb300.driver import cpe_grid
+    b.build()
+    rng = np.random.default_rng(19)
+    cr = gi.make_crystal(6, 4, 8, 4, NI, 30.0, qlist=[1])
+    gr = gi.make_grid(30.0, NT, NT, NT, ncont=64)
+    st = torch.cuda.Stream()
+    ctx = gw.GW(gr, cr, M=_c(rng, 1, 4, NI, 8, 8), stream=st)
+    n = 32
+    w = (2 * np.arange(64) + 1) * np.pi / 30.0
+    pole, res = rng.uniform(-1.0, 1.0, (2 * n, 3)), rng.uniform(0.05, 0.2, (2 * n, 3))
+    sig = torch.from_numpy((res[:, :, None] / (1j * w - pole[:, :, None])).sum(1)).cuda()
+    d = {k: torch.from_numpy(rng.uniform(-0.5, 0.5, 2 * n)).cuda() for k in ("eps", "sigx", "vxc")}
+    eqp, info = torch.zeros(2 * n, dtype=torch.float64, device="cuda"), torch.zeros(2 * n, dtype=torch.int32, device="cuda")
+    x = cpe_grid()
+    torch.cuda.synchronize()
+
+    def fit(m):
+        ctx.continue_(gw.GW_CPE, sig[:m], d["eps"][:m], d["sigx"][:m], d["vxc"][:m], None, None, eqp[:m], info[:m])
+
+    with torch.cuda.stream(st):
+        ctx.cpe_setup(x, 1e-3)
+        fit(n)
+        st.synchronize()
+        ref = eqp[:n].clone()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            fit(n)
+        ctx.cpe_setup(x[::2].copy(), 1e-4)
+        fit(2 * n)
+        st.synchronize()
+        eqp.fill_(float("nan"))
+        g.replay()
+        st.synchronize()
+        assert bool(torch.isfinite(ref).all()) and torch.equal(eqp[:n], ref)
+        ctx.sync()
+    ctx.close()
